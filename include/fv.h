@@ -388,9 +388,10 @@ fv_status fv_batch_set_schedule(fv_batch* h, fv_schedule schedule);
  * or 256: a CTA per patch), set per patch size p (1..max_patch_size).  The
  * default (also of launches without a plan) follows the patch size: 32
  * threads for up to 64 interior cells, 256 for 3D patches above 200 cells,
- * else 128; d = 1 supports 128 only (FV_ERR_UNSUPPORTED otherwise).
- * The mapping never changes the results (bitwise).  fv_batch_class_threads
- * reads the current choice.
+ * else 128; d = 1 supports 128 only (FV_ERR_UNSUPPORTED otherwise).  A launch
+ * of so few patches that this leaves most of the GPU idle takes up to 256
+ * threads a patch where no size was set.  The mapping never changes the
+ * results (bitwise).  fv_batch_class_threads reads the current choice.
  */
 fv_status fv_batch_set_class_threads(fv_batch* h, int p, int threads);
 fv_status fv_batch_class_threads(const fv_batch* h, int p, int* threads);

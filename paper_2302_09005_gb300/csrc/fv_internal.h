@@ -34,7 +34,7 @@ struct fv_batch {
   unsigned long long* d_partials = nullptr;  // FV_MAX_RED_BLOCKS slots
   double* d_sum_partials = nullptr;          // FV_MAX_RED_BLOCKS * 8 slots
   unsigned long long* d_queue = nullptr;     // FV_SCHED_QUEUE: positions handed out
-  int blocks_per_sm[3] = {0, 0, 0};          // occupancy by kernel mode (kModeUpdate..)
+  int blocks_per_sm[3][4] = {{0}};           // occupancy by kernel mode and CTA size
   // primitive carry of fv_run_steps: two buffers of prim_cap elements
   void* d_prim[2] = {nullptr, nullptr};
   int64_t prim_cap = 0;
@@ -138,6 +138,28 @@ inline int default_nt(int d, int p) {
   if (n <= 64) return 32;
   if (d == 3 && n > 200) return 256;
   return 128;
+}
+// Faces of a patch of size p.
+inline int64_t patch_faces(int d, int p) {
+  int64_t t = d;
+  for (int k = 1; k < d; ++k) t *= p;
+  return t * (p + 1);
+}
+// CTA size of an untuned launch of `count` patches: default_nt(), doubled
+// while the launch still fits once into 384 (FP64) or 128 (FP32) threads per
+// SM and a patch has faces for more lanes.  A small batch is one chain of a
+// patch's phases, and more warps shorten each phase: 64 patches of 8x8, FP64,
+// 50 steps in a graph 0.62 -> 0.44 ms (a warp -> eight per patch); updates of
+// 64 patches, FP64, 3^3 12.4 -> 8.2 us, 8x8 12.3 -> 8.2, 17x17 14.4 -> 12.4;
+// at 600 patches (beyond the line) a warp is as fast.  FP32 phases are short,
+// and past 128 threads per SM more warps cost more than they save (300
+// patches of 5^3: 6.4 us at 128 threads, 8.3 at 256).
+inline int untuned_nt(const fv_batch* h, int p, int64_t count) {
+  int nt = default_nt(h->d, p);
+  if (h->d == 1) return nt;
+  const int64_t room = (int64_t)h->num_sms * (h->prec == FV_FP64 ? 384 : 128);
+  while (nt < 256 && nt < patch_faces(h->d, p) && 2 * nt * count <= room) nt *= 2;
+  return nt;
 }
 // Per-precision, per-CTA-size launch and occupancy (fv_update.cu: double and
 // 128 threads; fv_update_f32.cu: float and 128; fv_update_nt.cu and

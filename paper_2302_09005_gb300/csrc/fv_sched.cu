@@ -89,7 +89,7 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
       }
       lc.nstage = stages_for(h, lc.pmax);
       const int pi = lc.pmax < 64 ? lc.pmax : 63;
-      lc.nt = h->cls_nt[pi] > 0 ? h->cls_nt[pi] : default_nt(h->d, lc.pmax);
+      lc.nt = h->cls_nt[pi] > 0 ? h->cls_nt[pi] : untuned_nt(h, lc.pmax, cnt);
       int& bps = h->occ_cache[f][pi][nt_index(lc.nt)];
       if (bps == 0) {
         cudaError_t e = step_occupancy(h, f, lc.pmax, lc.nstage, lc.nt, &bps);
@@ -108,8 +108,8 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
     cudaError_t e = launch_one_size(h, lu, l.n, &done);
     if (e != cudaSuccess || done) return e;
   }
-  l.nt = default_nt(h->d, h->max_patch_size);
-  int& bps = h->blocks_per_sm[f];
+  l.nt = untuned_nt(h, h->max_patch_size, l.n);
+  int& bps = h->blocks_per_sm[f][nt_index(l.nt)];
   if (bps == 0) {
     cudaError_t e = step_occupancy(h, f, h->max_patch_size, h->nstage, l.nt, &bps);
     if (e != cudaSuccess) return e;
