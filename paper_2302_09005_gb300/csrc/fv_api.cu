@@ -129,14 +129,6 @@ fv_status fv_batch_create(fv_batch** out, int d, int s, const fv_options* o, voi
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   h->smem_optin = smem_optin;
-#ifdef FV_FORCE_SINGLE_STAGE
-  h->nstage = 1;
-#else
-  h->nstage = 2;
-#endif
-  if (e == cudaSuccess &&
-      fv::update_smem_bytes(d, h->prec, h->max_patch_size, 2) > (size_t)smem_optin)
-    h->nstage = 1;
   if (e == cudaSuccess &&
       fv::update_smem_bytes(d, h->prec, h->max_patch_size, 1) > (size_t)smem_optin) {
     delete h;
@@ -160,11 +152,12 @@ fv_status fv_batch_create(fv_batch** out, int d, int s, const fv_options* o, voi
   h->d_queue = reinterpret_cast<unsigned long long*>(w + 192);
   h->d_partials = reinterpret_cast<unsigned long long*>(w + 256);
   h->d_sum_partials = reinterpret_cast<double*>(w + 256 + 8ull * FV_MAX_RED_BLOCKS);
-  // CTAs per SM of the untuned launches (their CTA size follows the patch size)
+  // stages and CTAs per SM of the untuned launches (their CTA size follows the
+  // patch size)
+  const int nt = fv::default_nt(d, h->max_patch_size), ni = fv::nt_index(nt);
   for (int mode = fv::kModeUpdate; mode <= fv::kModePrim && e == cudaSuccess; ++mode)
-    e = fv::step_occupancy(
-        h, mode, h->max_patch_size, h->nstage, fv::default_nt(d, h->max_patch_size),
-        &h->blocks_per_sm[mode][fv::nt_index(fv::default_nt(d, h->max_patch_size))]);
+    e = fv::step_shape(h, mode, h->max_patch_size, nt, &h->nstage[mode][ni],
+                       &h->blocks_per_sm[mode][ni]);
   if (e != cudaSuccess) {
     cudaFree(h->ws);
     delete h;

@@ -21,7 +21,7 @@ struct fv_batch {
   double gamma = 1.4;
   fv_precision prec = FV_FP64;
   int max_patch_size = 0;
-  int nstage = 2;  // shared-memory stages of the update kernel
+  int nstage[3][4] = {{0}};  // shared-memory stages of untuned launches, by kernel mode, CTA size
   cudaStream_t stream = nullptr;
   int device = 0;
   int num_sms = 0;
@@ -48,6 +48,7 @@ struct fv_batch {
   int cls_p[64] = {0};
   int64_t cls_begin[64] = {0}, cls_end[64] = {0};
   int occ_cache[3][64][4] = {{{0}}};         // CTAs per SM by (kernel mode, p, CTA size)
+  int stage_cache[3][64][4] = {{{0}}};       // and their shared-memory stages
   int cls_nt[64] = {0};                      // CTA size of the size-class launches (0: 128)
   int cls_only = -1;                         // autotuner: launch only this class (-1: all)
   int cls_real[64] = {0};                    // class c holds one valid size (not the rejects)
@@ -83,7 +84,7 @@ struct UpdateLaunch {
   int64_t corr_stride = 0;
   unsigned int* status = nullptr;
   bool fused = false;  // time-step mode: gather halos, dt from lam_in, reduce lam_next
-  int nstage = 0;      // shared-memory stages (0: the handle's)
+  int nstage = 2;      // shared-memory stages
   int nt = 128;        // threads per CTA
   const double* dx_patch = nullptr;  // update mode: per-patch cell sizes, or null
   double* dt_patch = nullptr;        // with dx_patch: per-patch dt (in, or out with local_cfl)
@@ -123,6 +124,9 @@ size_t update_smem_bytes(int d, fv_precision prec, int pmax, int nstage);
 cudaError_t launch_update(const fv_batch* h, const UpdateLaunch& a, int grid);
 cudaError_t step_occupancy(const fv_batch* h, int mode, int pmax, int nstage, int nt,
                            int* blocks_per_sm);
+// Shared-memory stages and resident CTAs per SM of a launch for patches up to
+// pmax with CTAs of nt threads.
+cudaError_t step_shape(const fv_batch* h, int mode, int pmax, int nt, int* nstage, int* bps);
 // Threads per CTA of the step kernel for one launch: 32, 64, 128 or 256.
 inline bool valid_nt(int nt) { return nt == 32 || nt == 64 || nt == 128 || nt == 256; }
 inline int nt_index(int nt) { return nt == 32 ? 0 : nt == 64 ? 1 : nt == 128 ? 2 : 3; }

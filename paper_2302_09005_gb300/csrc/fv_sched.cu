@@ -35,8 +35,20 @@ void plan_free(fv_batch* h) {
   h->ncls = 0;
 }
 
-static int stages_for(const fv_batch* h, int p) {
-  return update_smem_bytes(h->d, h->prec, p, 2) <= (size_t)h->smem_optin ? 2 : 1;
+// Two stages (the copy of the next patch runs under the current one) unless
+// one makes more CTAs resident: their number decides, since another CTA
+// computes while one waits for its copy (FP64 5^3 with the carry: 6.34 ms per
+// 262,144 patches with five one-stage CTAs per SM, 7.53 with three of two
+// stages).
+cudaError_t step_shape(const fv_batch* h, int mode, int pmax, int nt, int* nstage, int* bps) {
+  int one = 0, two = 0;
+  cudaError_t e = cudaSuccess;
+  if (update_smem_bytes(h->d, h->prec, pmax, 2) <= (size_t)h->smem_optin)
+    e = step_occupancy(h, mode, pmax, 2, nt, &two);
+  if (e == cudaSuccess) e = step_occupancy(h, mode, pmax, 1, nt, &one);
+  *nstage = one > two ? 1 : 2;
+  *bps = one > two ? one : two;
+  return e;
 }
 
 static int grid_for(const fv_batch* h, int64_t count, int bps) {
@@ -87,14 +99,15 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
         if (e != cudaSuccess) return e;
         if (done) continue;
       }
-      lc.nstage = stages_for(h, lc.pmax);
       const int pi = lc.pmax < 64 ? lc.pmax : 63;
       lc.nt = h->cls_nt[pi] > 0 ? h->cls_nt[pi] : untuned_nt(h, lc.pmax, cnt);
       int& bps = h->occ_cache[f][pi][nt_index(lc.nt)];
-      if (bps == 0) {
-        cudaError_t e = step_occupancy(h, f, lc.pmax, lc.nstage, lc.nt, &bps);
+      int& ns = h->stage_cache[f][pi][nt_index(lc.nt)];
+      if (bps == 0 || pi == 63) {  // slot 63: every size from 63 on
+        cudaError_t e = step_shape(h, f, lc.pmax, lc.nt, &ns, &bps);
         if (e != cudaSuccess) return e;
       }
+      lc.nstage = ns;
       cudaError_t e = launch_update(h, lc, grid_for(h, cnt, bps));
       if (e != cudaSuccess) return e;
     }
@@ -110,10 +123,12 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
   }
   l.nt = untuned_nt(h, h->max_patch_size, l.n);
   int& bps = h->blocks_per_sm[f][nt_index(l.nt)];
+  int& ns = h->nstage[f][nt_index(l.nt)];
   if (bps == 0) {
-    cudaError_t e = step_occupancy(h, f, h->max_patch_size, h->nstage, l.nt, &bps);
+    cudaError_t e = step_shape(h, f, h->max_patch_size, l.nt, &ns, &bps);
     if (e != cudaSuccess) return e;
   }
+  l.nstage = ns;
   if ((h->sched == FV_SCHED_LPT || h->sched == FV_SCHED_QUEUE) && plan_ok) {
     l.order = h->d_order;
     l.i_begin = 0;

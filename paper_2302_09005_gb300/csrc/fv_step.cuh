@@ -44,6 +44,7 @@
 #pragma once
 
 #include "fv_device.cuh"
+#include "fv_fxsum.cuh"
 #include "fv_internal.h"
 #include "fv_ptx.cuh"
 
@@ -416,6 +417,52 @@ __device__ __forceinline__ void mid_hook(const StepParams<T>& a, Pipe& pp,
   gather_dispatch<T, D, GATHER, PRIMIN, NT>(a, nx.p, nx.st, nx.fs);
 }
 
+// sum_k (G[j[k] + step] - G[j[k]]), the flux differences of one unknown of a
+// cell: FP32 one operation after the other; FP64 with d >= 2 as one
+// fixed-point sum on the integer pipe (fv_fxsum.cuh), where that is exact,
+// else one operation after the other too (in a loop: the compiler would run
+// predicated straight-line adds always, and it is the FP64 pipe that is to
+// be spared).
+template <int D>
+__device__ __forceinline__ float sum_diffs(const float* G, const int (&j)[D], int step,
+                                           const Arith<float>& ar) {
+  float acc = ar.sub(G[j[0] + step], G[j[0]]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) acc = ar.add(acc, ar.sub(G[j[k] + step], G[j[k]]));
+  return acc;
+}
+template <int D>
+__device__ __forceinline__ double sum_diffs(const double* G, const int (&j)[D], int step,
+                                            const Arith<double>& ar) {
+  if constexpr (D >= 2) {
+    uint32_t h[2 * D], l[2 * D], rh, rl;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const double gp = G[j[k] + step], gm = G[j[k]];
+      h[k] = (uint32_t)__double2hiint(gp);
+      l[k] = (uint32_t)__double2loint(gp);
+      h[D + k] = (uint32_t)__double2hiint(gm);
+      l[D + k] = (uint32_t)__double2loint(gm);
+    }
+    bool ok;
+    fx_sum<2 * D, D>(h, l, rh, rl, ok);
+    double r = __hiloint2double((int)rh, (int)rl);
+    if (!ok) {
+#pragma unroll 1
+      for (int k = 0; k < D; ++k) {
+        const int jk = k == 0 ? j[0] : (D == 3 && k == 2) ? j[D - 1] : j[1];
+        const double t = ar.sub(G[jk + step], G[jk]);
+        r = k == 0 ? t : ar.add(r, t);
+      }
+    }
+    return r;
+  }
+  double acc = ar.sub(G[j[0] + step], G[j[0]]);
+#pragma unroll
+  for (int k = 1; k < D; ++k) acc = ar.add(acc, ar.sub(G[j[k] + step], G[j[k]]));
+  return acc;
+}
+
 // ---------------------------------------------------------------------------
 // One patch: cells, faces, update.
 // ---------------------------------------------------------------------------
@@ -686,20 +733,13 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
       r /= p;
     }
     const int cid = g.cell(c);
-    T acc[S];
+    int jm[D];
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
-      const int jm = g.trans(c, k) + ptr * (c[k] - 1);
-      const T* Gk = G + k * S * nface;
-#pragma unroll
-      for (int v = 0; v < S; ++v) {
-        const T dG = ar.sub(Gk[v * nface + jm + ptr], Gk[v * nface + jm]);
-        acc[v] = k == 0 ? dG : ar.add(acc[v], dG);
-      }
-    }
+    for (int k = 0; k < D; ++k) jm[k] = g.trans(c, k) + ptr * (c[k] - 1) + k * S * nface;
     T qn[S];
 #pragma unroll
-    for (int v = 0; v < S; ++v) qn[v] = fma(mhr, acc[v], st[cid * S + v]);
+    for (int v = 0; v < S; ++v)
+      qn[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
     T* dst = dst_base + (int64_t)cid * S;
 #pragma unroll
     for (int v = 0; v < S; ++v) dst[v] = qn[v];
@@ -749,9 +789,13 @@ __device__ __forceinline__ void patch_dispatch(const StepParams<T>& a, int p, in
 }
 
 // Resident CTAs per SM the register allocation is sized for, given as the
-// resident threads per SM (3 CTAs of 128 threads for FP64, 6 for FP32).
+// resident threads per SM (5 CTAs of 128 threads for FP64, 6 for FP32).  FP64
+// at 5 (102 registers): the integer work of the update (fv_fxsum.cuh) runs
+// beside the FP64 work of the other resident CTAs, so more of them fill both
+// pipes (262,144 patches of 5^3 with the carry: 6.34 ms at 5 CTAs, 6.61 at 4,
+// 7.53 at 3; with the sums on the FP64 pipe 7.87 at 5 and 7.98 at 3).
 #ifndef FV_MINBLOCKS_FP64
-#define FV_MINBLOCKS_FP64 3
+#define FV_MINBLOCKS_FP64 5
 #endif
 #ifndef FV_MINBLOCKS_FP32
 #define FV_MINBLOCKS_FP32 6
@@ -937,7 +981,7 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
   a.n = l.n;
   a.n_elems = l.n_elems;
   a.pmax = l.pmax;
-  a.nstage = l.nstage > 0 ? l.nstage : h->nstage;
+  a.nstage = l.nstage;
   a.gamma = (T)l.gamma;
   a.gm1 = (T)(l.gamma - 1.0);
   a.dx = l.dx;
