@@ -565,8 +565,8 @@ fv_status fv_normalize_columns(float* x, int64_t rows, int cols, const float* mu
 
 /*
  * fv_conserved_totals -- FP64 sums over all interior cells of every unknown
- * (mass, momentum, energy), for conservation checks.  Fixed-order two-stage
- * reduction (per patch, then per block, then one block), so the result is
+ * (mass, momentum, energy), for conservation checks.  Fixed-order reduction
+ * (per patch, per slice of a chunk, per chunk, then the chunks), so the result is
  * bitwise reproducible.  FP32 handles accumulate in FP64.
  *   totals  device double[s].
  */
