@@ -257,6 +257,71 @@ __device__ __forceinline__ Prim<T, D> primitives(const T* q, T gm1, T gamma, boo
   return w;
 }
 
+// ---------------------------------------------------------------------------
+// FP32 bounds of an FP64 cell's wave speed, for maxima: only cells whose
+// upper bound reaches the largest lower bound can hold the maximum, and only
+// those need the FP64 primitives (19 operations on the scarce pipe; the
+// bounds cost none).  um is |u_k| (kdir = k) or the largest |u_k| (kdir < 0),
+// and lo <= um + c <= hi for the FP64 um + c; false (lo = 0, hi = inf) where
+// that cannot be told: values outside the floats' range, NaN, or a pressure
+// that is not certain to be positive -- the caller evaluates those cells.
+//
+// With x ~ y (1 +- 2^-23) for every truncated input and 2^-23 for the
+// approximate reciprocal, u is within 2^-21 of j / rho, the kinetic energy ke
+// within 2^-20, and (gamma - 1)(E - ke) within 2^-20 (E + ke) (gamma - 1) of
+// p; kWaveEps = 2^-18 covers these, the square root and the final sums four
+// times over.
+// ---------------------------------------------------------------------------
+constexpr float kWaveEps = 0x1p-18f;
+
+// |x| as a float, truncated; `ok` turns false outside the float range (zero
+// stays zero).
+__device__ __forceinline__ float mag_f32(double x, bool& ok) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7FFFFFFFu;
+  const unsigned l = (unsigned)__double2loint(x);
+  // exponents 2^-125 .. 2^126
+  const bool in = h - ((1023u - 125u) << 20) < (252u << 20);
+  const bool zero = (h | l) == 0u;
+  ok = ok && (in || zero);
+  const unsigned f = ((h << 3) | (l >> 29)) - (896u << 23);
+  return in ? __uint_as_float(f) : 0.f;
+}
+template <int D>
+__device__ __forceinline__ bool wave_bounds(const double* q, float gm1, float gamma, int kdir,
+                                            float& lo, float& hi) {
+  bool ok = __double2hiint(q[0]) > 0;  // rho > 0
+  const float rho = mag_f32(q[0], ok), E = mag_f32(q[D + 1], ok);
+  ok = ok && __double2hiint(q[D + 1]) > 0;
+  // far from the ends of the range, so that products neither overflow nor
+  // underflow where it matters
+  ok = ok && rho > 0x1p-60f && rho < 0x1p60f && E > 0x1p-60f && E < 0x1p60f;
+  float inv;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(rho));
+  float ke = 0.f, um = 0.f;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const float j = mag_f32(q[1 + k], ok), u = j * inv;
+    ke = fmaf(0.5f * j, u, ke);
+    um = (kdir < 0 || kdir == k) ? fmaxf(um, u) : um;
+  }
+  const float th = E - ke, tot = E + ke, g = gamma * gm1 * inv;
+  ok = ok && th > tot * kWaveEps;  // p > 0 for certain (false for NaN)
+  const float c2 = g * th, e2 = g * tot * kWaveEps;
+  float ch, cl;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(ch) : "f"(c2 + e2));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(cl) : "f"(fmaxf(c2 - e2, 0.f)));
+  hi = ok ? (um + ch) * (1.f + kWaveEps) : __int_as_float(0x7F800000);
+  lo = ok ? (um + cl) * (1.f - kWaveEps) : 0.f;
+  return ok;
+}
+// A float not above the wave speed x (a bit pattern of order_bits); 0 where
+// x has no float below it in range.
+__device__ __forceinline__ float wave_floor(unsigned long long x) {
+  bool ok = true;
+  const float f = mag_f32(__longlong_as_double((long long)x), ok);
+  return ok ? f : 0.f;
+}
+
 // Flux f^k (S = D + 2 values) and wave speed |u_k| + c of one cell (Eq. 2, 5).
 template <typename T, int D>
 __device__ __forceinline__ void flux_dir(const T* q, const Prim<T, D>& w, int k, T* f, T& lam) {
