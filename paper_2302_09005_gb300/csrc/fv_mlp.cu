@@ -111,28 +111,38 @@ __device__ __forceinline__ int prow(int t, int at, int c) {
   return (t >> 3) * kGroup + at + c * 128 + (t & 7) * 16;
 }
 
+// Four consecutive parameters (16-byte words where the vector is aligned).
+__device__ __forceinline__ float4 ld_par4(const float* p, bool vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ void st_bf16x4(unsigned char* dst, const float4& v) {
+  *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+}
+// A training step is a chain of two small kernels.  Each is launched while
+// the one before it still runs (programmatic dependent launch): it lets the
+// next one start, prepares what does not depend on the others, and waits here
+// until all of them are complete and their writes visible.  A step of 32,768
+// samples (256 tiles, one per CTA) is bound by the latency of that chain, not
+// by a unit: 35.5 us, with the parameters loaded one after the other, each
+// partial gradient's sum four loads deep and the loss summed by one thread;
+// 16.9 us with all loads of a phase in flight and the launches overlapped.
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <bool TRAIN>
 __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ alignas(8) uint64_t bar;
   __shared__ uint32_t tslot;
-  __shared__ float red[kRows];
+  __shared__ float red[kRows / 32];
   const int tid = threadIdx.x, warp = tid >> 5;
   float* bias = reinterpret_cast<float*>(sm + kBias);
 
-  // weights as BF16 K-major tiles; biases
-  for (int i = tid; i < 64 * 16; i += kRows)
-    *reinterpret_cast<uint16_t*>(sm + kW1 + kmajor(i >> 4, i & 15, 16)) =
-        f32_to_bf16(a.params[kOffW1 + i]);
-  for (int i = tid; i < 64 * 64; i += kRows)
-    *reinterpret_cast<uint16_t*>(sm + kW2 + kmajor(i >> 6, i & 63, 64)) =
-        f32_to_bf16(a.params[kOffW2 + i]);
-  for (int i = tid; i < 16 * 64; i += kRows)
-    *reinterpret_cast<uint16_t*>(sm + kW3 + kmajor(i >> 6, i & 63, 64)) =
-        i < 4 * 64 ? f32_to_bf16(a.params[kOffW3 + i]) : (uint16_t)0;
-  for (int i = tid; i < 132; i += kRows)
-    bias[i] = i < 64 ? a.params[kOffB1 + i]
-                     : (i < 128 ? a.params[kOffB2 + i - 64] : a.params[kOffB3 + i - 128]);
   if (TRAIN) {
     // the constant rows: ones at feature 80 of PC (B of GA) and at row 64 of
     // PB (A of GW3), zeros around them
@@ -157,6 +167,52 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     fence_mbar_init();
   }
   if (warp == 0) tc_alloc(&tslot, kTmemCols);
+  const int64_t ntiles = (a.rows + kRows - 1) / kRows;
+  float4 xv[4], tv = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto load_rows = [&](int64_t tile) {
+    const int64_t r = tile * kRows + tid;
+    const bool ok = tile < ntiles && r < a.rows;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      xv[i] = ok ? __ldg(reinterpret_cast<const float4*>(a.x + r * 16) + i)
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (TRAIN) tv = ok ? __ldg(reinterpret_cast<const float4*>(a.t + r * 4))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  load_rows(blockIdx.x);  // the samples are no kernel's output
+  grid_dep_wait();        // the parameters of the step before
+  grid_dep_launch();      // the update kernel may start its own preparations
+  {
+    // weights as BF16 K-major tiles, four of a row at a time, every load in
+    // flight before the first store; biases
+    const bool vec = ((uintptr_t)a.params & 15u) == 0;
+    float4 w1[2], w2[8], w3 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w2[i] = ld_par4(a.params + kOffW2 + 4 * (tid + i * kRows), vec);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) w1[i] = ld_par4(a.params + kOffW1 + 4 * (tid + i * kRows), vec);
+    if (tid < 64) w3 = ld_par4(a.params + kOffW3 + 4 * tid, vec);
+    const float bb = a.params[tid < 64 ? kOffB1 + tid : kOffB2 + tid - 64];
+    const float b3 = tid < 4 ? a.params[kOffB3 + tid] : 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = 4 * (tid + i * kRows);
+      st_bf16x4(sm + kW2 + kmajor(e >> 6, e & 63, 64), w2[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = 4 * (tid + i * kRows);
+      st_bf16x4(sm + kW1 + kmajor(e >> 4, e & 15, 16), w1[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {  // rows 4 .. 15 of W3 are zero
+      const int e = 4 * (tid + i * kRows);
+      st_bf16x4(sm + kW3 + kmajor(e >> 6, e & 63, 64),
+                e < 4 * 64 ? w3 : make_float4(0.f, 0.f, 0.f, 0.f));
+    }
+    bias[tid] = bb;
+    if (tid < 4) bias[128 + tid] = b3;
+  }
   fence_proxy_async_smem();
   tc_fence_before_sync();
   __syncthreads();
@@ -195,19 +251,6 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
                 tc_smem_desc(sm + kW1, 128, 256), idesc(kRows, 64, 0, 0), 0);
   };
 
-  const int64_t ntiles = (a.rows + kRows - 1) / kRows;
-  float4 xv[4], tv = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto load_rows = [&](int64_t tile) {
-    const int64_t r = tile * kRows + tid;
-    const bool ok = tile < ntiles && r < a.rows;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      xv[i] = ok ? __ldg(reinterpret_cast<const float4*>(a.x + r * 16) + i)
-                 : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (TRAIN) tv = ok ? __ldg(reinterpret_cast<const float4*>(a.t + r * 4))
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-  };
-  load_rows(blockIdx.x);
   float loss = 0.f;
   bool first = true;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -364,7 +407,9 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
           float v[16];
           tc_ld16(tGA + c, v);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) pg[kOffW2 + tid * 64 + c + i] = v[i];
+          for (int i = 0; i < 16; i += 4)
+            *reinterpret_cast<float4*>(pg + kOffW2 + tid * 64 + c + i) =
+                make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         }
         pg[kOffB2 + tid] = gb[0];
 #pragma unroll
@@ -374,7 +419,9 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
         tc_ld16(tGA + 64, v);
         const int h = tid - 64;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) pg[kOffW1 + h * 16 + i] = v[i];
+        for (int i = 0; i < 16; i += 4)
+          *reinterpret_cast<float4*>(pg + kOffW1 + h * 16 + i) =
+              make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         pg[kOffB1 + h] = gb[0];
         if (tid == 64) {
 #pragma unroll
@@ -382,13 +429,11 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
         }
       }
     }
-    red[tid] = loss;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, o);
+    if ((tid & 31) == 0) red[warp] = loss;
     __syncthreads();
-    if (tid == 0) {
-      float s = 0.f;
-      for (int i = 0; i < kRows; ++i) s += red[i];
-      a.part_loss[blockIdx.x] = s;
-    }
+    if (tid == 0) a.part_loss[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
   }
   if (failed) {
     if (tid == 0) atomicOr(a.status, ST_TIMEOUT);
@@ -424,20 +469,24 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(UpdateArgs u) {
   __shared__ float red[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
+  grid_dep_wait();    // the partial gradients
+  grid_dep_launch();  // the next step's network kernel may start
+  // Adam's state, loaded under the partials
+  const bool mine = w == 0 && i < kMlpParams && u.grad_out == nullptr;
+  const float m0 = mine ? u.m[i] : 0.f, v0 = mine ? u.v[i] : 0.f, p0 = mine ? u.params[i] : 0.f;
   float s = 0.f;
   if (i < kMlpParams) {
+    constexpr int kFly = 16;  // loads in flight, summed in order
+    const float* p = u.part + i;
     int c = w;
-    for (; c + 24 < u.nparts; c += 32) {  // four loads in flight, summed in order
-      const float v0 = u.part[(int64_t)c * kMlpParams + i];
-      const float v1 = u.part[(int64_t)(c + 8) * kMlpParams + i];
-      const float v2 = u.part[(int64_t)(c + 16) * kMlpParams + i];
-      const float v3 = u.part[(int64_t)(c + 24) * kMlpParams + i];
-      s += v0;
-      s += v1;
-      s += v2;
-      s += v3;
+    for (; c + 8 * (kFly - 1) < u.nparts; c += 8 * kFly) {
+      float v[kFly];
+#pragma unroll
+      for (int k = 0; k < kFly; ++k) v[k] = p[(int64_t)(c + 8 * k) * kMlpParams];
+#pragma unroll
+      for (int k = 0; k < kFly; ++k) s += v[k];
     }
-    for (; c < u.nparts; c += 8) s += u.part[(int64_t)c * kMlpParams + i];
+    for (; c < u.nparts; c += 8) s += p[(int64_t)c * kMlpParams];
   }
   red[w][lane] = s;
   __syncthreads();
@@ -448,17 +497,19 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(UpdateArgs u) {
     if (u.grad_out) {
       u.grad_out[i] = g;
     } else {
-      const float mi = u.b1 * u.m[i] + (1.f - u.b1) * g;
-      const float vi = u.b2 * u.v[i] + (1.f - u.b2) * g * g;
+      const float mi = u.b1 * m0 + (1.f - u.b1) * g;
+      const float vi = u.b2 * v0 + (1.f - u.b2) * g * g;
       u.m[i] = mi;
       u.v[i] = vi;
-      u.params[i] -= u.lr * (mi / u.c1) / (sqrtf(vi / u.c2) + u.eps);
+      u.params[i] = p0 - u.lr * (mi / u.c1) / (sqrtf(vi / u.c2) + u.eps);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 32 && u.loss_out) {
+  if (blockIdx.x == 0 && w == 1 && u.loss_out) {  // the loss, a lane per partial
     float l = 0.f;
-    for (int c = 0; c < u.nparts; ++c) l += u.part_loss[c];
-    *u.loss_out = l * u.inv_n;
+    for (int c = lane; c < u.nparts; c += 32) l += u.part_loss[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+    if (lane == 0) *u.loss_out = l * u.inv_n;
   }
 }
 
@@ -486,8 +537,27 @@ int mlp_grid(const fv_mlp_trainer* t, int64_t batch) {
   return (int)(tiles < t->grid_max ? tiles : t->grid_max);
 }
 
+// Launches a kernel of the chain; `early`: it may start while the kernel
+// before it on the stream, one of the chain too, still runs.
+template <typename K, typename A>
+cudaError_t launch_chain(K kernel, int grid, int threads, size_t smem, cudaStream_t stream,
+                         bool early, const A& args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 cudaError_t launch_net(const fv_mlp_trainer* t, bool train, const float* params, const float* x,
-                       const float* target, int64_t batch, float* y, int* grid_out) {
+                       const float* target, int64_t batch, float* y, int* grid_out,
+                       bool early) {
   fv::MlpArgs a;
   a.params = params;
   a.x = x;
@@ -500,11 +570,8 @@ cudaError_t launch_net(const fv_mlp_trainer* t, bool train, const float* params,
   a.status = t->status;
   const int grid = mlp_grid(t, batch);
   if (grid_out) *grid_out = grid;
-  if (train)
-    fv::mlp_kernel<true><<<grid, fv::kRows, fv::kSmemBytes, t->stream>>>(a);
-  else
-    fv::mlp_kernel<false><<<grid, fv::kRows, fv::kSmemBytes, t->stream>>>(a);
-  return cudaGetLastError();
+  return launch_chain(train ? fv::mlp_kernel<true> : fv::mlp_kernel<false>, grid, fv::kRows,
+                      fv::kSmemBytes, t->stream, early, a);
 }
 
 cudaError_t launch_update(const fv_mlp_trainer* t, int nparts, int64_t batch, float* grad_out,
@@ -525,8 +592,8 @@ cudaError_t launch_update(const fv_mlp_trainer* t, int nparts, int64_t batch, fl
   u.c1 = grad_out ? 1.f : 1.f - powf(u.b1, (float)step);
   u.c2 = grad_out ? 1.f : 1.f - powf(u.b2, (float)step);
   u.loss_out = loss;
-  fv::mlp_update_kernel<<<(fv::kMlpParams + 31) / 32, 256, 0, t->stream>>>(u);
-  return cudaGetLastError();
+  return launch_chain(fv::mlp_update_kernel, (fv::kMlpParams + 31) / 32, 256, 0, t->stream, true,
+                      u);
 }
 
 }  // namespace
@@ -603,7 +670,7 @@ fv_status fv_mlp_forward(fv_mlp_trainer* t, const float* params, const float* x,
                          float* y) {
   if (!t || !params || !x || !y || batch < 1 || batch > t->max_batch) return FV_ERR_INVALID_ARG;
   if (((uintptr_t)x | (uintptr_t)y) & 15u) return FV_ERR_ALIGNMENT;
-  cudaError_t e = launch_net(t, false, params, x, nullptr, batch, y, nullptr);
+  cudaError_t e = launch_net(t, false, params, x, nullptr, batch, y, nullptr, false);
   return e == cudaSuccess ? FV_OK : FV_ERR_CUDA;
 }
 
@@ -613,7 +680,7 @@ fv_status fv_mlp_grad(fv_mlp_trainer* t, const float* params, const float* x,
     return FV_ERR_INVALID_ARG;
   if (((uintptr_t)x | (uintptr_t)target) & 15u) return FV_ERR_ALIGNMENT;
   int grid = 0;
-  cudaError_t e = launch_net(t, true, params, x, target, batch, nullptr, &grid);
+  cudaError_t e = launch_net(t, true, params, x, target, batch, nullptr, &grid, false);
   if (e == cudaSuccess) e = launch_update(t, grid, batch, grad, nullptr, 0.f, 1, loss);
   return e == cudaSuccess ? FV_OK : FV_ERR_CUDA;
 }
@@ -636,7 +703,7 @@ fv_status fv_mlp_train_steps(fv_mlp_trainer* t, float* params, const float* x,
     const int step = first_step + k;
     const int64_t r0 = ((int64_t)(step - 1) % nb) * batch;
     int grid = 0;
-    e = launch_net(t, true, params, x + r0 * 16, target + r0 * 4, batch, nullptr, &grid);
+    e = launch_net(t, true, params, x + r0 * 16, target + r0 * 4, batch, nullptr, &grid, k > 0);
     if (e == cudaSuccess)
       e = launch_update(t, grid, batch, nullptr, params, lr, step, losses ? losses + k : nullptr);
   }
