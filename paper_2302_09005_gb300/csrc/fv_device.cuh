@@ -151,57 +151,55 @@ __device__ __forceinline__ Arith<T> plain_arith() {
 // ---------------------------------------------------------------------------
 // Reciprocal and square root, once per cell of the interior and face halo.
 //
-// FP64 is the scarce unit on GB300 (two FP64 lanes per SM), so the FP64
-// forms refine a cheap seed with FMAs instead of running the full IEEE
-// division and square root sequences:
-//   1/a     Newton-Raphson in its cubic form: with y0 ~ 1/a and
-//           e = 1 - a y0, 1/a = y0 / (1 - e) = y0 (1 + e + e^2 + ...), so
-//           y = y0 + y0 (e + e^2) leaves a relative error of order e^3;
-//   sqrt(x) with r0 ~ x^(-1/2), s0 = x r0 and e = 1 - s0 r0 = 1 - x r0^2,
-//           sqrt(x) = s0 (1 - e)^(-1/2) = s0 (1 + e/2 + 3e^2/8 + ...),
-//           truncated after the e^2 term (binomial series).
-// The seeds come from the FP32 special-function unit, not from the f64
-// approximation instructions (which spend FP64 operations of their own): the
-// double's sign, exponent and leading 20 fraction bits are repacked as a
-// float with integer operations, the float reciprocal / reciprocal square
-// root is taken, and the result is repacked as a double.  The seed is good
-// to about 2^-20, so the cubic step leaves ~2^-60 for 1/a and the two-term
-// series ~2^-62 for sqrt: within an ulp or two of the correctly rounded
-// result (measured by fv_selftest_math against the IEEE operations), far
-// inside the 1e-12 tolerance of the update.  Arguments outside the float
-// exponent range (and zero, negative, non-finite values) take the IEEE
-// operation.  The FP32 forms are the special-function unit's approximations
-// themselves (one instruction each, within about an ulp and two ulps): the
-// FP32 path is bound by instruction issue, where the IEEE sequences cost
-// about ten instructions per cell each, and its error target (1e-5 after a
-// step) is far above an ulp of FP32.
+// FP64 is the scarce unit on GB300 (two FP64 lanes per SM), so the FP64 forms
+// spend two FP64 operations each, on the last Newton step; everything before
+// it runs in FP32 and integers, on pipes the FP64 kernels leave idle.  The
+// argument's significand is split exactly into two floats fh + fl (fl up to
+// bits of relative weight 2^-46); a float seed from the special-function
+// unit gets a float correction from its residual, which FP32 fused
+// multiply-adds give to all its bits:
+//   1/a      y0 ~ 1/fh, e = 1 - fh y0 - fl y0, d = y0 (e + e^2);
+//   sqrt(x)  s ~ fh rsqrt(fh), e = fh - s s + fl, d = e rsqrt(fh) / 2;
+// and seed + d, added in integers on the double's fraction bits, is good to
+// about 2^-42.  The FP64 step squares that:
+//   y + y (1 - a y)   and   s + (x - s^2) h,  h = rsqrt(fh)/2 ~ 1/(2s),
+// each with one rounding of consequence: within an ulp of the correctly
+// rounded result (measured by fv_selftest_math against the IEEE operations).
+// The forms they replace refined the bare float seed with three and five FP64
+// operations.  Arguments whose result or steps would leave the normal range
+// (and zero, negative, non-finite values) take the IEEE operation.  The FP32
+// forms are the special-function unit's approximations themselves (one
+// instruction each, within about an ulp and two ulps): the FP32 path is bound
+// by instruction issue, where the IEEE sequences cost about ten instructions
+// per cell each, and its error target (1e-5 after a step) is far above an ulp
+// of FP32.
 // ---------------------------------------------------------------------------
 
-// Double -> float carrying the double's leading 20 fraction bits (truncated);
-// false if the exponent does not fit a normal float with margin.
-__device__ __forceinline__ bool f64_seed_as_f32(double x, float& f) {
-  const unsigned hi = (unsigned)__double2hiint(x);
-  const int ef = (int)((hi >> 20) & 0x7FFu) - 1023 + 127;
-  if ((hi >> 31) != 0u || ef < 4 || ef > 250) return false;
-  f = __uint_as_float(((unsigned)ef << 23) | ((hi & 0xFFFFFu) << 3));
-  return true;
-}
-// Exact float -> double by repacking the fields (positive normal floats).
-__device__ __forceinline__ double f32_as_f64(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned e = ((b >> 23) & 0xFFu) - 127u + 1023u;
-  return __hiloint2double((int)((e << 20) | ((b & 0x7FFFFFu) >> 3)), (int)((b & 7u) << 29));
+// x (a float in [1/2, 2], as a double) + n 2^-53 x's binade below 1, 2^-52
+// from 1 on: n is added to the double's bit pattern.
+__device__ __forceinline__ void add_units(float x, long long n, unsigned& hi, unsigned& lo) {
+  const unsigned b = __float_as_uint(x);
+  const unsigned long long v =
+      (((unsigned long long)((b >> 3) + (896u << 20)) << 32) | (b << 29)) + (unsigned long long)n;
+  hi = (unsigned)(v >> 32);
+  lo = (unsigned)v;
 }
 
 __device__ __forceinline__ double recip(double a, const Arith<double>& ar = plain_arith<double>()) {
-  float f;
-  if (!f64_seed_as_f32(a, f)) return 1.0 / a;
-  float rf;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-  const double y = f32_as_f64(rf);
-  const double e = fma(neg_t(a), y, 1.0);
-  const double t = fma(e, e, e);
-  return fma(y, t, y);
+  const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
+  if ((hi >> 20) - 2u > 2042u) return 1.0 / a;  // sign clear, exponent 2 .. 2044
+  const float fh = __uint_as_float(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+  const float fl = __uint_as_float(0x34000000u | ((lo >> 6) & 0x7FFFFFu)) - 0x1p-23f;
+  float y0;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(fh));
+  y0 = fminf(fmaxf(y0, 0.5f), 1.0f);
+  const float e = fmaf(-fl, y0, fmaf(-fh, y0, 1.0f));
+  const float d = y0 * fmaf(e, e, e);
+  unsigned yh, yl;
+  add_units(y0, (long long)__float2int_rn(d * 0x1p52f) * 2, yh, yl);
+  yh += (1023u << 20) - (hi & 0x7FF00000u);
+  const double y = __hiloint2double((int)yh, (int)yl);
+  return fma(y, fma(neg_t(a), y, 1.0), y);
 }
 __device__ __forceinline__ float recip(float a, const Arith<float>& = plain_arith<float>()) {
   float r;
@@ -210,15 +208,25 @@ __device__ __forceinline__ float recip(float a, const Arith<float>& = plain_arit
 }
 
 __device__ __forceinline__ double sqrt_t(double x, const Arith<double>& ar = plain_arith<double>()) {
-  float f;
-  if (!f64_seed_as_f32(x, f)) return sqrt(x);
-  float rf;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-  const double r = f32_as_f64(rf);
-  const double s0 = ar.mul(x, r);
-  const double e = fma(neg_t(s0), r, 1.0);
-  const double t = ar.mul(e, fma(e, 0.375, 0.5));
-  return fma(s0, t, s0);
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if ((hi >> 20) - 64u > 1982u) return sqrt(x);  // exponent 64 .. 2046
+  // x = f 4^k with f in [1, 4)
+  const unsigned odd = ((hi >> 20) & 1u) ^ 1u;
+  const int k = ((int)(hi >> 20) - 1023 - (int)odd) >> 1;
+  const unsigned ob = odd << 23;
+  const float fh = __uint_as_float((0x3F800000u + ob) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+  const float fl = __uint_as_float((0x34000000u + ob) | ((lo >> 6) & 0x7FFFFFu)) -
+                   __uint_as_float(0x34000000u + ob);
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fh));
+  const float s = fminf(fmaxf(fh * r, 1.0f), 2.0f);
+  const float d = (fmaf(-s, s, fh) + fl) * (0.5f * r);
+  unsigned sh, sl;
+  add_units(s, (long long)__float2int_rn(d * 0x1p51f) * 2, sh, sl);
+  const double s0 = __hiloint2double((int)(sh + ((unsigned)k << 20)), (int)sl);
+  const unsigned rb = __float_as_uint(r);
+  const double h = __hiloint2double((int)((rb >> 3) + ((unsigned)(895 - k) << 20)), (int)(rb << 29));
+  return fma(fma(neg_t(s0), s0, x), h, s0);
 }
 __device__ __forceinline__ float sqrt_t(float x, const Arith<float>& = plain_arith<float>()) {
   float r;
