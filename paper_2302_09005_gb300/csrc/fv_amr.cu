@@ -38,27 +38,71 @@ struct fv_amr_plan {
 
 namespace fv {
 
-template <typename T>
-__global__ void amr_halo_kernel(T* __restrict__ q, const int64_t* __restrict__ dst,
-                                const int64_t* __restrict__ start,
-                                const int64_t* __restrict__ src, const int32_t* __restrict__ neg,
-                                int64_t ncell, int s) {
+// Bound by the latency of its dependent loads (the plan's entry, then the
+// sources): a cell's S unknowns are loaded together, and a restricted cell
+// keeps eight of its sources in flight (they are added in the plan's order
+// all the same).  With the unknowns in a loop of runtime length, their sums
+// were in local memory (22,933 patches of 5^3 on two levels: FP64 260 -> 217 us,
+// FP32 189 -> 163).
+template <typename T, int S>
+__global__ void __launch_bounds__(256) amr_halo_kernel(
+    T* __restrict__ q, const int64_t* __restrict__ dst, const int64_t* __restrict__ start,
+    const int64_t* __restrict__ src, const int32_t* __restrict__ neg, int64_t ncell) {
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell;
        c += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = start[c], e = start[c + 1];
+    const int64_t b = start[c], e = start[c + 1], d = dst[c];
     const int ng = neg[c];
-    T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
-    for (int64_t j = b; j < e; ++j) {
-      const T* v = q + src[j];
-      for (int u = 0; u < s; ++u) acc[u] += v[u];
+    T acc[S];
+    if (e - b == 1) {
+      const T* v = q + src[b];
+#pragma unroll
+      for (int u = 0; u < S; ++u) acc[u] = v[u];
+    } else {
+#pragma unroll
+      for (int u = 0; u < S; ++u) acc[u] = T(0);
+      constexpr int kFly = 8;
+      int64_t j = b;
+      for (; j + kFly <= e; j += kFly) {
+        T v[kFly][S];
+#pragma unroll
+        for (int m = 0; m < kFly; ++m) {
+          const T* p = q + src[j + m];
+#pragma unroll
+          for (int u = 0; u < S; ++u) v[m][u] = p[u];
+        }
+#pragma unroll
+        for (int m = 0; m < kFly; ++m)
+#pragma unroll
+          for (int u = 0; u < S; ++u) acc[u] += v[m][u];
+      }
+      for (; j < e; ++j) {
+        const T* p = q + src[j];
+#pragma unroll
+        for (int u = 0; u < S; ++u) acc[u] += p[u];
+      }
+      const T cnt = (T)(e - b);
+#pragma unroll
+      for (int u = 0; u < S; ++u) acc[u] = acc[u] / cnt;
     }
-    const int64_t cnt = e - b;
-    T* o = q + dst[c];
-    for (int u = 0; u < s; ++u) {
-      T val = cnt == 1 ? acc[u] : acc[u] / (T)cnt;
-      o[u] = (u == ng) ? -val : val;
-    }
+    T* o = q + d;
+#pragma unroll
+    for (int u = 0; u < S; ++u) o[u] = (u == ng) ? -acc[u] : acc[u];
   }
+}
+
+template <typename T, int S>
+static void launch_amr_t(const fv_batch* h, const fv_amr_plan* pl, void* q, int grid) {
+  amr_halo_kernel<T, S><<<grid, 256, 0, h->stream>>>(static_cast<T*>(q), pl->d_dst, pl->d_start,
+                                                     pl->d_src, pl->d_neg, pl->ncell);
+}
+template <typename T>
+static void launch_amr(const fv_batch* h, const fv_amr_plan* pl, void* q, int grid) {
+  if (pl->s == 3)
+    launch_amr_t<T, 3>(h, pl, q, grid);
+  else if (pl->s == 4)
+    launch_amr_t<T, 4>(h, pl, q, grid);
+  else
+    launch_amr_t<T, 5>(h, pl, q, grid);
 }
 
 }  // namespace fv
@@ -259,11 +303,9 @@ fv_status fv_amr_halo_fill(fv_batch* h, const fv_amr_plan* pl, void* q) {
   const int64_t want = (pl->ncell + 255) / 256;
   const int grid = (int)(want < (int64_t)h->num_sms * 8 ? want : (int64_t)h->num_sms * 8);
   if (h->prec == FV_FP64)
-    fv::amr_halo_kernel<double><<<grid, 256, 0, h->stream>>>(
-        static_cast<double*>(q), pl->d_dst, pl->d_start, pl->d_src, pl->d_neg, pl->ncell, pl->s);
+    fv::launch_amr<double>(h, pl, q, grid);
   else
-    fv::amr_halo_kernel<float><<<grid, 256, 0, h->stream>>>(
-        static_cast<float*>(q), pl->d_dst, pl->d_start, pl->d_src, pl->d_neg, pl->ncell, pl->s);
+    fv::launch_amr<float>(h, pl, q, grid);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? FV_OK : amr_err(h, FV_ERR_CUDA, cudaGetErrorString(e));
 }
