@@ -155,7 +155,8 @@ fv_status fv_batch_create(fv_batch** out, int d, int s, const fv_options* o, voi
   // stages and CTAs per SM of the untuned launches (their CTA size follows the
   // patch size)
   const int nt = fv::default_nt(d, h->max_patch_size), ni = fv::nt_index(nt);
-  for (int mode = fv::kModeUpdate; mode <= fv::kModePrim && e == cudaSuccess; ++mode)
+  const int modes = opt.precision == FV_FP64 ? 4 : 3;
+  for (int mode = fv::kModeUpdate; mode < modes && e == cudaSuccess; ++mode)
     e = fv::step_shape(h, mode, h->max_patch_size, nt, &h->nstage[mode][ni],
                        &h->blocks_per_sm[mode][ni]);
   if (e != cudaSuccess) {
@@ -378,13 +379,13 @@ fv_status fv_patch_sums(fv_batch* h, const void* q, const int64_t* off, const in
 static fv_status time_step_impl(fv_batch* h, const void* in, void* out, const int64_t* off,
                                 const int32_t* sizes, const int32_t* nbr, int64_t n, double dx,
                                 double cfl, double* lambda_patch, const float* corr,
-                                const void* prim_in, void* prim_out);
+                                const void* prim_in, void* prim_out, bool own);
 
 fv_status fv_time_step(fv_batch* h, const void* in, void* out, const int64_t* off,
                        const int32_t* sizes, const int32_t* nbr, int64_t n, double dx,
                        double cfl, double* lambda_patch) {
   return time_step_impl(h, in, out, off, sizes, nbr, n, dx, cfl, lambda_patch, nullptr, nullptr,
-                        nullptr);
+                        nullptr, false);
 }
 
 fv_status fv_prim_stride(const fv_batch* h, int64_t* elems_per_patch) {
@@ -398,7 +399,7 @@ fv_status fv_time_step_prim(fv_batch* h, const void* in, void* out, const void* 
                             const int32_t* nbr, int64_t n, double dx, double cfl,
                             double* lambda_patch) {
   return time_step_impl(h, in, out, off, sizes, nbr, n, dx, cfl, lambda_patch, nullptr, prim_in,
-                        prim_out);
+                        prim_out, false);
 }
 
 fv_status fv_time_step_corrected(fv_batch* h, const void* in, void* out, const int64_t* off,
@@ -407,13 +408,14 @@ fv_status fv_time_step_corrected(fv_batch* h, const void* in, void* out, const i
   if (!h) return FV_ERR_INVALID_ARG;
   if (!corr) return set_err(h, FV_ERR_INVALID_ARG, "null corrections");
   if (h->d != 2) return set_err(h, FV_ERR_UNSUPPORTED, "corrections are 2D");
-  return time_step_impl(h, in, out, off, sizes, nbr, n, dx, cfl, nullptr, corr, nullptr, nullptr);
+  return time_step_impl(h, in, out, off, sizes, nbr, n, dx, cfl, nullptr, corr, nullptr, nullptr,
+                        false);
 }
 
 static fv_status time_step_impl(fv_batch* h, const void* in, void* out, const int64_t* off,
                                 const int32_t* sizes, const int32_t* nbr, int64_t n, double dx,
                                 double cfl, double* lambda_patch, const float* corr,
-                                const void* prim_in, void* prim_out) {
+                                const void* prim_in, void* prim_out, bool own) {
   if (!h) return FV_ERR_INVALID_ARG;
   h->last_error[0] = 0;
   if (!(dx > 0.0) || !(cfl > 0.0)) return set_err(h, FV_ERR_INVALID_ARG, "dx, cfl must be > 0");
@@ -451,7 +453,8 @@ static fv_status time_step_impl(fv_batch* h, const void* in, void* out, const in
   l.corr_stride = 2ll * 4 * (h->max_patch_size + 1) * h->max_patch_size;
   l.prim_in = prim_in;
   l.prim_out = prim_out;
-  l.prim_stride = fv::prim_stride_elems(h->d, h->prec, h->max_patch_size);
+  l.prim_stride = fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, own);
+  l.prim_own = own;
   e = fv::launch_scheduled(h, l);
   if (e != cudaSuccess) return cuda_err(h, e, "time step kernel");
   h->lam_cur = nxt;
@@ -472,7 +475,7 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
   const bool carry = h->prec == FV_FP64 && n_steps > 1;
   if (carry && n > 0) {
     const size_t es = h->prec == FV_FP64 ? 8 : 4;
-    const int64_t need = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size);
+    const int64_t need = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, true);
     if (need > h->prim_cap) {
       cudaError_t e = cudaStreamSynchronize(h->stream);
       graph_cache_clear(h);
@@ -497,7 +500,8 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
       // step k reads the primitives step k-1 left and hands on its own
       const void* pin = (!carry || k == 0) ? nullptr : h->d_prim[(k - 1) & 1];
       void* pout = (carry && k + 1 < n_steps) ? h->d_prim[k & 1] : nullptr;
-      s = time_step_impl(h, a, b, off, sizes, nbr, n, dx, cfl, nullptr, nullptr, pin, pout);
+      s = time_step_impl(h, a, b, off, sizes, nbr, n, dx, cfl, nullptr, nullptr, pin, pout,
+                         carry);
       std::swap(a, b);
     }
     return s;

@@ -21,7 +21,7 @@ struct fv_batch {
   double gamma = 1.4;
   fv_precision prec = FV_FP64;
   int max_patch_size = 0;
-  int nstage[3][4] = {{0}};  // shared-memory stages of untuned launches, by kernel mode, CTA size
+  int nstage[4][4] = {{0}};  // shared-memory stages of untuned launches, by kernel mode, CTA size
   cudaStream_t stream = nullptr;
   int device = 0;
   int num_sms = 0;
@@ -34,7 +34,7 @@ struct fv_batch {
   unsigned long long* d_partials = nullptr;  // FV_MAX_RED_BLOCKS slots
   double* d_sum_partials = nullptr;          // FV_MAX_RED_BLOCKS * 8 slots
   unsigned long long* d_queue = nullptr;     // FV_SCHED_QUEUE: positions handed out
-  int blocks_per_sm[3][4] = {{0}};           // occupancy by kernel mode and CTA size
+  int blocks_per_sm[4][4] = {{0}};           // occupancy by kernel mode and CTA size
   // primitive carry of fv_run_steps: two buffers of prim_cap elements
   void* d_prim[2] = {nullptr, nullptr};
   int64_t prim_cap = 0;
@@ -47,8 +47,8 @@ struct fv_batch {
   int ncls = 0;
   int cls_p[64] = {0};
   int64_t cls_begin[64] = {0}, cls_end[64] = {0};
-  int occ_cache[3][64][4] = {{{0}}};         // CTAs per SM by (kernel mode, p, CTA size)
-  int stage_cache[3][64][4] = {{{0}}};       // and their shared-memory stages
+  int occ_cache[4][64][4] = {{{0}}};         // CTAs per SM by (kernel mode, p, CTA size)
+  int stage_cache[4][64][4] = {{{0}}};       // and their shared-memory stages
   int cls_nt[64] = {0};                      // CTA size of the size-class launches (0: 128)
   int cls_only = -1;                         // autotuner: launch only this class (-1: all)
   int cls_real[64] = {0};                    // class c holds one valid size (not the rejects)
@@ -92,23 +92,29 @@ struct UpdateLaunch {
   const void* prim_in = nullptr;  // time step: carried primitives of `in`, or null
   void* prim_out = nullptr;       // time step: primitives of `out`, or null
   int64_t prim_stride = 0;        // elements per patch of the primitive buffers
+  bool prim_own = false;          // FP64: both in fv_run_steps' own form
   int uniform_p = 0;              // every patch of the launch has this size (0: unknown)
   unsigned long long* queue = nullptr;  // zeroed counter: CTAs pop positions (null: stride)
 };
 
 // Kernel modes: update (halos filled by the caller), time step (halo gather,
-// CFL from the device, next-step maximum), time step with primitive carry.
+// CFL from the device, next-step maximum), time step with primitive carry in
+// the documented form, and in fv_run_steps' own form (FP64).
 constexpr int kModeUpdate = 0;
 constexpr int kModeStep = 1;
 constexpr int kModePrim = 2;
+constexpr int kModeOwn = 3;
 inline int step_mode(const UpdateLaunch& l) {
-  return !l.fused ? kModeUpdate : (l.prim_in != nullptr ? kModePrim : kModeStep);
+  if (!l.fused) return kModeUpdate;
+  if (l.prim_in == nullptr) return kModeStep;
+  return l.prim_own ? kModeOwn : kModePrim;
 }
 
 // Elements per patch of a primitive buffer: (d + 3) p^d for p = pmax, rounded
-// up to 16 bytes.
-inline int64_t prim_stride_elems(int d, fv_precision prec, int pmax) {
-  int64_t c = d + 3;
+// up to 16 bytes; 2d + 1 components in fv_run_steps' own form (u, p and the
+// wave speeds |u_k| + c).
+inline int64_t prim_stride_elems(int d, fv_precision prec, int pmax, bool own = false) {
+  int64_t c = own ? 2 * d + 1 : d + 3;
   for (int k = 0; k < d; ++k) c *= pmax;
   const int64_t vec = prec == FV_FP64 ? 2 : 4;
   return (c + vec - 1) / vec * vec;

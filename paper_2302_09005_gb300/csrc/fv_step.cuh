@@ -79,6 +79,7 @@ struct StepParams {
   int local_cfl;           // with dx_patch: dt_i = cfl dx_i / (d lambda_i) per patch
   const T* __restrict__ prim_in;  // carried primitives of `in` (primitive-carry mode)
   T* __restrict__ prim_out;       // primitives of `out` (time-step modes), or null
+  int prim_own;                   // FP64: prim_out in the library's own form (kCarryOwn)
   int64_t prim_stride;            // elements per patch of prim_in / prim_out
   long long wait_limit = FV_WAIT_LIMIT;  // cycles of a wait for a patch's copy
   unsigned long long* queue = nullptr;    // zeroed counter of positions handed out, or null
@@ -93,15 +94,41 @@ template <int D>
 __host__ __device__ inline int stage_elems(int p) {
   return ipow_d<D>(p + 2) * (D + 2);
 }
-// interior primitives: D+3 components (u_1..u_D, p, c, E+p) of p^D cells
-template <int D>
-__host__ __device__ inline int iprim_elems(int p) {
-  return (D + 3) * ipow_d<D>(p);
+// How a launch gets the primitives of its input: computed from the state, from
+// a caller's carry in the documented form (u_1..u_D, p, c, E+p), or from
+// fv_run_steps' own buffers in the form the FP64 kernel works with.
+constexpr int kCarryNone = 0, kCarryDoc = 1, kCarryOwn = 2;
+// Interior primitives, components of p^D cells: in FP64 u_1..u_D, p and the
+// wave speeds |u_k| + c, k = 1..D, which every face of direction k takes from
+// its two cells (one addition a cell and direction where its two faces took
+// two each, and E + p is not needed at all); in FP32, and in the documented
+// carry, u_1..u_D, p, c, E+p.  With it the time step without the carry skips
+// the new state's primitives where they cannot raise the CFL maximum (see the
+// epilogue).  Measured with both: 20 steps of 200,000 uneven patches 95.3 ->
+// 88.7 ms, 9,177 6^3 patches' engine loop 667 -> 650 us, learned step 315 ->
+// 300 us, refined mesh 909 -> 879 us; the documented carry (energy flux without
+// E + p only) 6.25 -> 6.19 ms.
+template <typename T, int CARRY>
+constexpr bool kLamForm() {
+  return sizeof(T) == 8 && CARRY != kCarryDoc;
 }
-// face-halo primitives: 2D faces x 4 components (u_normal, p, c, E+p) x p^(D-1)
-template <int D>
+template <typename T, int D, int CARRY>
+__host__ __device__ constexpr int prim_comps() {
+  return kLamForm<T, CARRY>() ? 2 * D + 1 : D + 3;
+}
+template <typename T, int D, int CARRY>
+__host__ __device__ inline int iprim_elems(int p) {
+  return prim_comps<T, D, CARRY>() * ipow_d<D>(p);
+}
+// Face-halo primitives: 2D faces x (u_normal, p, |u_normal| + c) in FP64
+// (c in the documented carry), (u_normal, p, c, E+p) in FP32 x p^(D-1).
+template <typename T>
+__host__ __device__ constexpr int halo_comps() {
+  return sizeof(T) == 8 ? 3 : 4;
+}
+template <typename T, int D>
 __host__ __device__ inline int hprim_elems(int p) {
-  return 2 * D * 4 * (ipow_d<D>(p) / p);
+  return 2 * D * halo_comps<T>() * (ipow_d<D>(p) / p);
 }
 // face fluxes G: D directions x (D+2) unknowns x (p+1) p^(D-1) faces
 template <int D>
@@ -134,12 +161,14 @@ struct FaceSrc {
 // Threads per CTA the kernel is built for: one CTA advances one patch at a
 // time; small patches use a warp or two, the largest eight warps.
 constexpr int kMaxNT = 256;
-// Shared-memory header: two mbarriers (16 B), per-warp reduction slots, and
-// the face sources of the two stages (2 x 6 x 24 B).
+// Shared-memory header: two mbarriers (16 B), per-warp reduction slots, the
+// CTA's largest new wave speed so far (8 B), and the face sources of the two
+// stages (2 x 6 x 24 B).
 constexpr int kRedOff = 16;
+constexpr int kRunMaxOff = kRedOff + 8 * (kMaxNT / 32);
 constexpr int kFaceSrcOff = 128;
 constexpr int kHdrBytes = 512;
-static_assert(kRedOff + 8 * (kMaxNT / 32) <= kFaceSrcOff, "header too small");
+static_assert(kRunMaxOff + 8 <= kFaceSrcOff, "header too small");
 static_assert(kFaceSrcOff + 2 * 6 * (int)sizeof(FaceSrc) <= kHdrBytes, "header too small");
 
 // Shared-memory carve-up for patches up to pmax (element counts of T).  A
@@ -148,16 +177,16 @@ static_assert(kFaceSrcOff + 2 * 6 * (int)sizeof(FaceSrc) <= kHdrBytes, "header t
 // the current one (one stage when two do not fit: the copy of the next
 // patch then starts after the current patch is done).  The face fluxes G
 // follow the stages.
-template <int D>
+template <typename T, int D, int CARRY>
 struct Carve {
   int nstage, box, ip, hp, stage, g;
-  __host__ __device__ Carve(int pmax, int vec, int nstage_)
+  __host__ __device__ Carve(int pmax, int nstage_)
       : nstage(nstage_),
-        box(round_up(stage_elems<D>(pmax), vec)),
-        ip(round_up(iprim_elems<D>(pmax), vec)),
-        hp(round_up(hprim_elems<D>(pmax), vec)),
+        box(round_up(stage_elems<D>(pmax), 16 / sizeof(T))),
+        ip(round_up(iprim_elems<T, D, CARRY>(pmax), 16 / sizeof(T))),
+        hp(round_up(hprim_elems<T, D>(pmax), 16 / sizeof(T))),
         stage(box + ip + hp),
-        g(round_up(gface_elems<D>(pmax), vec)) {}
+        g(round_up(gface_elems<D>(pmax), 16 / sizeof(T))) {}
   __host__ __device__ int total() const { return nstage * stage + g; }
 };
 
@@ -203,16 +232,16 @@ __device__ __forceinline__ bool patch_ok(const StepParams<T>& a, int64_t j, int&
 // and, carrying primitives, of its interior primitive block.  The state's
 // ragged tail (< 16 bytes) lies in the last cell of the patch, a corner
 // (d >= 2, never read) or the +x halo cell (d = 1, gathered separately).
-template <typename T, int D, bool PRIMIN>
+template <typename T, int D, int CARRY>
 __device__ __forceinline__ void issue_stage(const StepParams<T>& a, int64_t pid, int pj,
                                             int64_t offj, const Stage<T>& st, uint64_t* bar) {
   const uint32_t bytes = (uint32_t)(stage_elems<D>(pj) * sizeof(T)) & ~15u;
   uint32_t pbytes = 0;
-  if constexpr (PRIMIN) pbytes = (uint32_t)round_up(iprim_elems<D>(pj) * (int)sizeof(T), 16);
+  if constexpr (CARRY != kCarryNone) pbytes = (uint32_t)round_up(iprim_elems<T, D, CARRY>(pj) * (int)sizeof(T), 16);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   mbar_arrive_expect_tx(bar, bytes + pbytes);
   bulk_copy_g2s(st.box, a.in + offj, bytes, bar);
-  if constexpr (PRIMIN) bulk_copy_g2s(st.ip, a.prim_in + pid * a.prim_stride, pbytes, bar);
+  if constexpr (CARRY != kCarryNone) bulk_copy_g2s(st.ip, a.prim_in + pid * a.prim_stride, pbytes, bar);
 }
 
 // The source of the halo cells of face f of patch j (the neighbour table and
@@ -287,7 +316,7 @@ __host__ __device__ constexpr bool kGatherSlots() {
 // copies (a wall's negated normal momentum with a plain load and store); when
 // primitives are carried, also the face-halo primitives (u_normal, p, c,
 // E + p) from the sources' carried blocks (a wall negates u_normal).
-template <typename T, int D, int P, bool GATHER, bool PRIMIN, int NT>
+template <typename T, int D, int P, bool GATHER, int CARRY, int NT>
 __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, const Stage<T>& s,
                                             const FaceSrc* fs) {
   if constexpr (!GATHER && D != 1) return;
@@ -301,14 +330,14 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
     const int cs = g.cell_kt(k, m.ck, r);
     T* dst = s.box + cd * S;
     const T* src = a.in + m.off + (int64_t)cs * S;
-    T* pd = s.hp + f * 4 * ptr + r;
+    T* pd = s.hp + f * halo_comps<T>() * ptr + r;
     const T* ps = nullptr;
-    if constexpr (PRIMIN)
+    if constexpr (CARRY != kCarryNone)
       ps = a.prim_in + (int64_t)m.pidx * a.prim_stride + g.icell_kt(k, m.ck - 1, r);
     if (!m.neg) {
 #pragma unroll
       for (int v = 0; v < S; ++v) cp_async_elem(dst + v, src + v);
-      if constexpr (PRIMIN) cp_async_elem(pd, ps + k * g.nint());
+      if constexpr (CARRY != kCarryNone) cp_async_elem(pd, ps + k * g.nint());
     } else {  // wall: the normal momentum and velocity mirrored
 #pragma unroll
       for (int v = 0; v < S; ++v) {
@@ -317,11 +346,12 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
         else
           cp_async_elem(dst + v, src + v);
       }
-      if constexpr (PRIMIN) pd[0] = neg_t(__ldg(ps + k * g.nint()));
+      if constexpr (CARRY != kCarryNone) pd[0] = neg_t(__ldg(ps + k * g.nint()));
     }
-    if constexpr (PRIMIN) {
-#pragma unroll
-      for (int v = 1; v < 4; ++v) cp_async_elem(pd + v * ptr, ps + (D + v - 1) * g.nint());
+    if constexpr (CARRY != kCarryNone) {
+      cp_async_elem(pd + ptr, ps + D * g.nint());
+      cp_async_elem(pd + 2 * ptr, ps + (D + 1 + (kLamForm<T, CARRY>() ? k : 0)) * g.nint());
+      if constexpr (halo_comps<T>() == 4) cp_async_elem(pd + 3 * ptr, ps + (D + 2) * g.nint());
     }
   };
   if constexpr (kGatherSlots<D, P, NT>()) {
@@ -364,19 +394,19 @@ __host__ __device__ constexpr bool specialised(int p) {
   return D == 3 ? (p == 3 || p == 5 || p == 7) : (p == 3 || p == 5 || p == 8 || p == 17);
 }
 
-template <typename T, int D, bool GATHER, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, int CARRY, int NT>
 __device__ __forceinline__ void gather_dispatch(const StepParams<T>& a, int pj,
                                                 const Stage<T>& s, const FaceSrc* fs) {
   if constexpr (!GATHER && D != 1) return;
 #define FV_GH(PP)                                                               \
   if constexpr (specialised<D, NT>(PP)) {                                       \
-    if (pj == PP) return gather_halo<T, D, PP, GATHER, PRIMIN, NT>(a, pj, s, fs); \
+    if (pj == PP) return gather_halo<T, D, PP, GATHER, CARRY, NT>(a, pj, s, fs); \
   }
   FV_GH(3)
   FV_GH(5)
   FV_GH(7)
   FV_GH(8)
-  gather_halo<T, D, 0, GATHER, PRIMIN, NT>(a, pj, s, fs);
+  gather_halo<T, D, 0, GATHER, CARRY, NT>(a, pj, s, fs);
 #undef FV_GH
 }
 
@@ -401,7 +431,7 @@ struct NextPatch {
 
 // Inside a patch, after a barrier: wait for the bulk copy of the next patch
 // and start its halo gather, so both overlap the rest of this patch.
-template <typename T, int D, bool GATHER, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, int CARRY, int NT>
 __device__ __forceinline__ void mid_hook(const StepParams<T>& a, Pipe& pp,
                                          const NextPatch<T>& nx) {
   if (nx.j >= a.i_end) return;
@@ -414,7 +444,7 @@ __device__ __forceinline__ void mid_hook(const StepParams<T>& a, Pipe& pp,
     pp.timeout = true;
     return;
   }
-  gather_dispatch<T, D, GATHER, PRIMIN, NT>(a, nx.p, nx.st, nx.fs);
+  gather_dispatch<T, D, GATHER, CARRY, NT>(a, nx.p, nx.st, nx.fs);
 }
 
 // sum_k (G[j[k] + step] - G[j[k]]), the flux differences of one unknown of a
@@ -493,10 +523,11 @@ __host__ __device__ constexpr bool kWarpSlots() {
   }
 }
 
-template <typename T, int D, int P, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, int P, bool GATHER, bool FUSED, int CARRY, int NT>
 __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, int64_t i,
                                               int64_t off, const Stage<T>& cur, T* G, T mhr,
                                               unsigned long long* red,
+                                              unsigned long long* run_max,
                                               unsigned long long& lam_next, Pipe& pp,
                                               const NextPatch<T>& nx) {
   constexpr int S = D + 2;
@@ -511,7 +542,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
   bool bad = false;
 
   // ---- cells: primitives of the interior and face-halo cells ---------------
-  if constexpr (!PRIMIN) {
+  if constexpr (CARRY == kCarryNone) {
     const int nint_pad = (nint + 31) & ~31;
     const int nA = nint_pad + 2 * D * ptr;
     FV_PRAGMA_UNROLL(FV_UNROLL_CELLS)
@@ -532,8 +563,13 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
         for (int m = 0; m < D; ++m) ip[m * nint + t] = w.u[m];
         ip[D * nint + t] = w.p;
-        ip[(D + 1) * nint + t] = w.c;
-        ip[(D + 2) * nint + t] = w.ep;
+        if constexpr (kLamForm<T, CARRY>()) {
+#pragma unroll
+          for (int m = 0; m < D; ++m) ip[(D + 1 + m) * nint + t] = ar.add(abs_t(w.u[m]), w.c);
+        } else {
+          ip[(D + 1) * nint + t] = w.c;
+          ip[(D + 2) * nint + t] = w.ep;
+        }
       } else if (t >= nint_pad) {
         const int hc = t - nint_pad;
         const int f = hc / ptr;
@@ -547,21 +583,27 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
         T uk = w.u[0];
 #pragma unroll
         for (int m = 1; m < D; ++m) uk = (k == m) ? w.u[m] : uk;
-        T* h = hp + f * 4 * ptr + r;
+        T* h = hp + f * halo_comps<T>() * ptr + r;
         h[0] = uk;
         h[ptr] = w.p;
-        h[2 * ptr] = w.c;
-        h[3 * ptr] = w.ep;
+        if constexpr (kLamForm<T, CARRY>()) {
+          h[2 * ptr] = ar.add(abs_t(uk), w.c);
+        } else {
+          h[2 * ptr] = w.c;
+          h[3 * ptr] = w.ep;
+        }
       }
     }
     __syncthreads();
-    mid_hook<T, D, GATHER, PRIMIN, NT>(a, pp, nx);
+    mid_hook<T, D, GATHER, CARRY, NT>(a, pp, nx);
   }
 
   // ---- faces: G = f_L + f_R - a (Q_R - Q_L), once per face -------------------
   // Cell b (halo-inclusive, 0..p+1) along k at transverse index tr: its state
   // and the primitives of direction k (face-halo block at the patch
   // boundary, interior block inside).
+  // FP64: c is the wave speed |u| + c (the sound speed in the documented
+  // carry), e unused.
   struct CellK {
     T q[S];
     T u, pr, c, e;
@@ -575,25 +617,27 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     for (int v = 0; v < S; ++v) x.q[v] = st[cid * S + v];
     const bool h0 = lo && b == 0, h1 = hi && b == p + 1;
     const int ic = g.icell_kt(k, h0 ? 0 : (h1 ? p - 1 : b - 1), tr);
-    const T* pu = h0 ? hp + 8 * k * ptr + tr
-                     : (h1 ? hp + (8 * k + 4) * ptr + tr : ip + k * nint + ic);
-    const T* pp_ = h0 ? hp + (8 * k + 1) * ptr + tr
-                      : (h1 ? hp + (8 * k + 5) * ptr + tr : ip + D * nint + ic);
-    const int sp = (h0 || h1) ? ptr : nint;
+    constexpr int HC = halo_comps<T>();
+    const T* h = hp + ((2 * k + (h1 ? 1 : 0)) * HC) * ptr + tr;
+    const T* pu = (h0 || h1) ? h : ip + k * nint + ic;
+    const T* pp_ = (h0 || h1) ? h + ptr : ip + D * nint + ic;
+    const int sp = (h0 || h1) ? ptr : nint * (kLamForm<T, CARRY>() ? k + 1 : 1);
     x.u = pu[0];
     x.pr = pp_[0];
     x.c = pp_[sp];
-    x.e = pp_[2 * sp];
+    if constexpr (HC == 4) x.e = pp_[2 * sp];
   };
   // The flux of face j (k) between cells L and R, stored into G.
   auto flux = [&](const int k, const int j, const CellK& L, const CellK& R,
                   unsigned long long& lmax) {
-    const T uL = L.u, pL = L.pr, cL = L.c, eL = L.e;
-    const T uR = R.u, pR = R.pr, cR = R.c, eR = R.e;
+    const T uL = L.u, pL = L.pr, cL = L.c;
+    const T uR = R.u, pR = R.pr, cR = R.c;
     const T* qL = L.q;
     const T* qR = R.q;
     // a = max(|u_k| + c) over the two cells (Eq. 5)
-    const T am = max_by_bits(ar.add(abs_t(uL), cL), ar.add(abs_t(uR), cR));
+    const T am = kLamForm<T, CARRY>()
+                     ? max_by_bits(cL, cR)
+                     : max_by_bits(ar.add(abs_t(uL), cL), ar.add(abs_t(uR), cR));
     const unsigned long long ab = order_bits(am);
     lmax = ab > lmax ? ab : lmax;
     // G = f_L + f_R - a (Q_R - Q_L) = (f_L + a Q_L) + (f_R - a Q_R).  The
@@ -602,7 +646,9 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     // f + a Q folds to Q (u_k + a) (+ p): with s_L = u_L + a, s_R = u_R - a,
     //   G_rho = rho_L s_L + rho_R s_R,
     //   G_m   = j_mL s_L + j_mR s_R + (p_L + p_R) [m = k],
-    //   G_E   = (E + p)_L u_L + (E + p)_R u_R + a (E_L - E_R).
+    //   G_E   = E_L s_L + E_R s_R + p_L u_L + p_R u_R                     (FP64)
+    //         = (E + p)_L u_L + (E + p)_R u_R + a (E_L - E_R)             (FP32),
+    // four operations either way.
     const T sL = ar.add(uL, am), sR = ar.sub(uR, am);
     const T ps = ar.add(pL, pR);
     T gs[S];
@@ -610,7 +656,10 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
     for (int m = 0; m < D; ++m)
       gs[1 + m] = fma(qL[1 + m], sL, fma(qR[1 + m], sR, (m == k) ? ps : T(-0.0)));
-    gs[D + 1] = fma(am, ar.sub(qL[D + 1], qR[D + 1]), fma(eL, uL, ar.mul(eR, uR)));
+    if constexpr (sizeof(T) == 8)
+      gs[D + 1] = fma(qL[D + 1], sL, fma(qR[D + 1], sR, fma(pL, uL, ar.mul(pR, uR))));
+    else
+      gs[D + 1] = fma(am, ar.sub(qL[D + 1], qR[D + 1]), fma(L.e, uL, ar.mul(R.e, uR)));
     T* Gk = G + k * S * nface;
 #pragma unroll
     for (int v = 0; v < S; ++v) {
@@ -700,7 +749,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     if ((tid & 31) == 0) red[tid >> 5] = lmax;
   }
   __syncthreads();
-  if constexpr (PRIMIN) mid_hook<T, D, GATHER, PRIMIN, NT>(a, pp, nx);
+  if constexpr (CARRY != kCarryNone) mid_hook<T, D, GATHER, CARRY, NT>(a, pp, nx);
   unsigned long long lam_bits = 0ull;
   if (want_lam) {
     lam_bits = red[0];
@@ -724,6 +773,8 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 
   // ---- update: Q - (dt/2dx) sum_k (G_+ - G_-) -----------------------------------
   T* dst_base = a.out + off;
+  float run_floor = 0.f;
+  if constexpr (FUSED && sizeof(T) == 8) run_floor = wave_floor(*run_max);
   for (int t = tid; t < nint; t += NT) {
     int c[3] = {0, 0, 0};
     int r = t;
@@ -744,21 +795,55 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
     for (int v = 0; v < S; ++v) dst[v] = qn[v];
     if constexpr (FUSED) {
-      // primitives and wave speed of the new state, for the next step's CFL
-      // condition (and its primitive carry)
-      const Prim<T, D> w = primitives<T, D>(qn, a.gm1, a.gamma, bad, ar);
+      // the new state's wave speed, for the next step's CFL condition, and
+      // its primitives, for the carry
+      T* po = a.prim_out != nullptr ? a.prim_out + i * a.prim_stride + t : nullptr;
+      if constexpr (sizeof(T) == 4) {
+        const Prim<T, D> w = primitives<T, D>(qn, a.gm1, a.gamma, bad, ar);
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const unsigned long long lb = order_bits(ar.add(abs_t(w.u[k]), w.c));
-        lam_next = lb > lam_next ? lb : lam_next;
-      }
-      if (a.prim_out != nullptr) {
-        T* po = a.prim_out + i * a.prim_stride + t;
+        for (int k = 0; k < D; ++k) {
+          const unsigned long long lb = order_bits(ar.add(abs_t(w.u[k]), w.c));
+          lam_next = lb > lam_next ? lb : lam_next;
+        }
+        if (po != nullptr) {
 #pragma unroll
-        for (int m = 0; m < D; ++m) po[m * nint] = w.u[m];
-        po[D * nint] = w.p;
-        po[(D + 1) * nint] = w.c;
-        po[(D + 2) * nint] = w.ep;
+          for (int m = 0; m < D; ++m) po[m * nint] = w.u[m];
+          po[D * nint] = w.p;
+          po[(D + 1) * nint] = w.c;
+          po[(D + 2) * nint] = w.ep;
+        }
+      } else {
+        // FP64: a cell whose wave speed is certain to lie below one already
+        // met by the CTA (wave_bounds) needs no primitives for the maximum;
+        // where the carry wants them anyway, the bounds would cost more
+        // integer work than the sums they save
+        float lo, hi;
+        if (po != nullptr ||
+            !wave_bounds<D>(qn, (float)a.gm1, (float)a.gamma, -1, lo, hi) || hi >= run_floor) {
+          const Prim<T, D> w = primitives<T, D>(qn, a.gm1, a.gamma, bad, ar);
+          T lam[D];
+          unsigned long long m = 0ull;
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            lam[k] = ar.add(abs_t(w.u[k]), w.c);
+            const unsigned long long lb = order_bits(lam[k]);
+            m = lb > m ? lb : m;
+          }
+          if (po == nullptr && m > lam_next) atomicMax(run_max, m);
+          lam_next = m > lam_next ? m : lam_next;
+          if (po != nullptr) {
+#pragma unroll
+            for (int m = 0; m < D; ++m) po[m * nint] = w.u[m];
+            po[D * nint] = w.p;
+            if (a.prim_own) {
+#pragma unroll
+              for (int m = 0; m < D; ++m) po[(D + 1 + m) * nint] = lam[m];
+            } else {
+              po[(D + 1) * nint] = w.c;
+              po[(D + 2) * nint] = w.ep;
+            }
+          }
+        }
       }
     }
   }
@@ -766,25 +851,26 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
   if (bad) atomicOr(a.status, ST_NONPHYSICAL);
 }
 
-template <typename T, int D, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 __device__ __forceinline__ void patch_dispatch(const StepParams<T>& a, int p, int64_t i,
                                                int64_t off, const Stage<T>& st, T* G, T hr,
                                                unsigned long long* red,
+                                               unsigned long long* run_max,
                                                unsigned long long& lam_next, Pipe& pp,
                                                const NextPatch<T>& nx) {
 #define FV_PC(PP)                                                                           \
   if constexpr (specialised<D, NT>(PP)) {                                                   \
     if (p == PP)                                                                            \
-      return patch_compute<T, D, PP, GATHER, FUSED, PRIMIN, NT>(a, p, i, off, st, G, hr, red, \
-                                                                lam_next, pp, nx);          \
+      return patch_compute<T, D, PP, GATHER, FUSED, CARRY, NT>(a, p, i, off, st, G, hr, red, \
+                                                                run_max, lam_next, pp, nx); \
   }
   FV_PC(3)
   FV_PC(5)
   FV_PC(7)
   FV_PC(8)
   FV_PC(17)
-  patch_compute<T, D, 0, GATHER, FUSED, PRIMIN, NT>(a, p, i, off, st, G, hr, red, lam_next, pp,
-                                                    nx);
+  patch_compute<T, D, 0, GATHER, FUSED, CARRY, NT>(a, p, i, off, st, G, hr, red, run_max,
+                                                    lam_next, pp, nx);
 #undef FV_PC
 }
 
@@ -806,16 +892,16 @@ constexpr int min_blocks() {
   return threads / NT > 0 ? threads / NT : 1;
 }
 
-template <typename T, int D, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
     step_kernel(StepParams<T> a) {
-  static_assert(!PRIMIN || (GATHER && FUSED), "the primitive carry is a time-step mode");
+  static_assert(CARRY == kCarryNone || (GATHER && FUSED), "the primitive carry is a time-step mode");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   unsigned long long* red = reinterpret_cast<unsigned long long*>(smem_raw + kRedOff);
+  unsigned long long* run_max = reinterpret_cast<unsigned long long*>(smem_raw + kRunMaxOff);
   FaceSrc* fsrc = reinterpret_cast<FaceSrc*>(smem_raw + kFaceSrcOff);  // [stage][face]
-  constexpr int VEC = 16 / sizeof(T);
-  const Carve<D> cv(a.pmax, VEC, a.nstage);
+  const Carve<T, D, CARRY> cv(a.pmax, a.nstage);
   const bool single = a.nstage == 1;
   T* const sbase = reinterpret_cast<T*>(smem_raw + kHdrBytes);
   // stage s (0 or 1; the same one when single), built by arithmetic so the
@@ -840,6 +926,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+    *run_max = 0ull;
     fence_mbar_init();
   }
   __syncthreads();
@@ -873,14 +960,14 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
   int s = 0;
   if (cur < a.i_end) {
     face_sources<T, D, GATHER>(a, pidc, pc, oc, fsrc);
-    if (tid == 0) issue_stage<T, D, PRIMIN>(a, pidc, pc, oc, stage_at(0), &bar[0]);
+    if (tid == 0) issue_stage<T, D, CARRY>(a, pidc, pc, oc, stage_at(0), &bar[0]);
     pp.pending = 1u;
     __syncthreads();  // face sources visible
     const bool ok = wait_patch_copy(&bar[0], 0u, a.wait_limit);
     if (ok) {
       pp.parity ^= 1u;
       pp.pending = 0u;
-      gather_dispatch<T, D, GATHER, PRIMIN, NT>(a, pc, stage_at(0), fsrc);
+      gather_dispatch<T, D, GATHER, CARRY, NT>(a, pc, stage_at(0), fsrc);
     } else {
       pp.timeout = true;
     }
@@ -903,17 +990,17 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
     if (single) {
       nx_mid.j = a.i_end;  // the one stage is busy until this patch is done
     } else if (nx.j < a.i_end) {
-      if (tid == 0) issue_stage<T, D, PRIMIN>(a, nx.pid, nx.p, nx.off, nx.st, &bar[nx.slot]);
+      if (tid == 0) issue_stage<T, D, CARRY>(a, nx.pid, nx.p, nx.off, nx.st, &bar[nx.slot]);
       pp.pending |= 1u << nx.slot;
     }
-    patch_dispatch<T, D, GATHER, FUSED, PRIMIN, NT>(a, pc, pidc, oc, stage_at(s), G, hr, red,
-                                                    lam_next, pp, nx_mid);
+    patch_dispatch<T, D, GATHER, FUSED, CARRY, NT>(a, pc, pidc, oc, stage_at(s), G, hr, red,
+                                                    run_max, lam_next, pp, nx_mid);
     cp_async_wait_all();
     if (__syncthreads_or(pp.timeout)) break;
     if (single && nx.j < a.i_end) {
-      if (tid == 0) issue_stage<T, D, PRIMIN>(a, nx.pid, nx.p, nx.off, nx.st, &bar[0]);
+      if (tid == 0) issue_stage<T, D, CARRY>(a, nx.pid, nx.p, nx.off, nx.st, &bar[0]);
       pp.pending |= 1u;
-      mid_hook<T, D, GATHER, PRIMIN, NT>(a, pp, nx);
+      mid_hook<T, D, GATHER, CARRY, NT>(a, pp, nx);
       cp_async_wait_all();
       if (__syncthreads_or(pp.timeout)) break;
     }
@@ -946,14 +1033,14 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
 }
 
 // Bytes of dynamic shared memory of the kernel for patches up to pmax.
-template <int D>
-inline size_t step_smem_bytes(int es, int pmax, int nstage) {
-  return kHdrBytes + (size_t)es * Carve<D>(pmax, 16 / es, nstage).total();
+template <typename T, int D, int CARRY>
+inline size_t step_smem_bytes(int pmax, int nstage) {
+  return kHdrBytes + sizeof(T) * (size_t)Carve<T, D, CARRY>(pmax, nstage).total();
 }
 
 // Raises the kernel's dynamic shared-memory limit on the current device once
 // (not per launch, so launches can be captured into CUDA graphs).
-template <typename T, int D, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 static cudaError_t ensure_smem(size_t smem) {
   static int set_bytes[64] = {0};
   std::lock_guard<std::mutex> lock(smem_attr_mutex());
@@ -961,13 +1048,13 @@ static cudaError_t ensure_smem(size_t smem) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && set_bytes[dev] >= (int)smem) return cudaSuccess;
-  e = cudaFuncSetAttribute(step_kernel<T, D, GATHER, FUSED, PRIMIN, NT>,
+  e = cudaFuncSetAttribute(step_kernel<T, D, GATHER, FUSED, CARRY, NT>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess && dev >= 0 && dev < 64) set_bytes[dev] = (int)smem;
   return e;
 }
 
-template <typename T, int D, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int grid) {
   StepParams<T> a;
   a.in = static_cast<const T*>(l.in);
@@ -1004,28 +1091,29 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
   a.prim_in = static_cast<const T*>(l.prim_in);
   a.prim_out = static_cast<T*>(l.prim_out);
   a.prim_stride = l.prim_stride;
+  a.prim_own = l.prim_own ? 1 : 0;
   a.wait_limit = h->wait_limit;
   a.queue = l.queue;
-  const size_t smem = step_smem_bytes<D>((int)sizeof(T), l.pmax, a.nstage);
-  cudaError_t e = ensure_smem<T, D, GATHER, FUSED, PRIMIN, NT>(smem);
+  const size_t smem = step_smem_bytes<T, D, CARRY>(l.pmax, a.nstage);
+  cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
-  step_kernel<T, D, GATHER, FUSED, PRIMIN, NT><<<grid, NT, smem, h->stream>>>(a);
+  step_kernel<T, D, GATHER, FUSED, CARRY, NT><<<grid, NT, smem, h->stream>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, int D, bool GATHER, bool FUSED, bool PRIMIN, int NT>
+template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 static cudaError_t occupancy_t(int pmax, int nstage, int* bps) {
-  const size_t smem = step_smem_bytes<D>((int)sizeof(T), pmax, nstage);
-  cudaError_t e = ensure_smem<T, D, GATHER, FUSED, PRIMIN, NT>(smem);
+  const size_t smem = step_smem_bytes<T, D, CARRY>(pmax, nstage);
+  cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      bps, step_kernel<T, D, GATHER, FUSED, PRIMIN, NT>, NT, smem);
+      bps, step_kernel<T, D, GATHER, FUSED, CARRY, NT>, NT, smem);
 }
 
 // Launch / occupancy of one precision and CTA size, dispatched over d and
 // the mode (explicitly instantiated in the fv_update*.cu translation units).
 // d = 1 is built for 128 threads only.
-template <typename T, int NT, bool G_, bool F_, bool P_>
+template <typename T, int NT, bool G_, bool F_, int P_>
 static cudaError_t launch_by_d(const fv_batch* h, const UpdateLaunch& l, int grid) {
   if (h->d == 2) return launch_step_t<T, 2, G_, F_, P_, NT>(h, l, grid);
   if (h->d == 3) return launch_step_t<T, 3, G_, F_, P_, NT>(h, l, grid);
@@ -1033,7 +1121,7 @@ static cudaError_t launch_by_d(const fv_batch* h, const UpdateLaunch& l, int gri
   return cudaErrorInvalidConfiguration;
 }
 
-template <typename T, int NT, bool G_, bool F_, bool P_>
+template <typename T, int NT, bool G_, bool F_, int P_>
 static cudaError_t occupancy_by_d(int d, int pmax, int nstage, int* bps) {
   if (d == 2) return occupancy_t<T, 2, G_, F_, P_, NT>(pmax, nstage, bps);
   if (d == 3) return occupancy_t<T, 3, G_, F_, P_, NT>(pmax, nstage, bps);
@@ -1044,16 +1132,25 @@ static cudaError_t occupancy_by_d(int d, int pmax, int nstage, int* bps) {
 template <typename T, int NT>
 cudaError_t launch_step_nt(const fv_batch* h, const UpdateLaunch& l, int grid) {
   const int mode = step_mode(l);
-  if (mode == kModePrim) return launch_by_d<T, NT, true, true, true>(h, l, grid);
-  if (mode == kModeStep) return launch_by_d<T, NT, true, true, false>(h, l, grid);
-  return launch_by_d<T, NT, false, false, false>(h, l, grid);
+  if (mode == kModePrim) return launch_by_d<T, NT, true, true, kCarryDoc>(h, l, grid);
+  if (mode == kModeStep) return launch_by_d<T, NT, true, true, kCarryNone>(h, l, grid);
+  if (mode == kModeOwn) {  // fv_run_steps carries in FP64 only
+    if constexpr (sizeof(T) == 8) return launch_by_d<T, NT, true, true, kCarryOwn>(h, l, grid);
+    return cudaErrorInvalidConfiguration;
+  }
+  return launch_by_d<T, NT, false, false, kCarryNone>(h, l, grid);
 }
 
 template <typename T, int NT>
 cudaError_t occupancy_nt(int d, int mode, int pmax, int nstage, int* bps) {
-  if (mode == kModePrim) return occupancy_by_d<T, NT, true, true, true>(d, pmax, nstage, bps);
-  if (mode == kModeStep) return occupancy_by_d<T, NT, true, true, false>(d, pmax, nstage, bps);
-  return occupancy_by_d<T, NT, false, false, false>(d, pmax, nstage, bps);
+  if (mode == kModePrim) return occupancy_by_d<T, NT, true, true, kCarryDoc>(d, pmax, nstage, bps);
+  if (mode == kModeStep) return occupancy_by_d<T, NT, true, true, kCarryNone>(d, pmax, nstage, bps);
+  if (mode == kModeOwn) {
+    if constexpr (sizeof(T) == 8)
+      return occupancy_by_d<T, NT, true, true, kCarryOwn>(d, pmax, nstage, bps);
+    return cudaErrorInvalidConfiguration;
+  }
+  return occupancy_by_d<T, NT, false, false, kCarryNone>(d, pmax, nstage, bps);
 }
 
 }  // namespace fv

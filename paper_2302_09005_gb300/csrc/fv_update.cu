@@ -22,11 +22,21 @@ FV_EXTERN(float, 64)
 FV_EXTERN(float, 256)
 #undef FV_EXTERN
 
+template <int D>
+static size_t smem_by_prec(fv_precision prec, int pmax, int nstage) {
+  // the larger of the FP64 modes' forms
+  if (prec == FV_FP64) {
+    const size_t a = step_smem_bytes<double, D, kCarryNone>(pmax, nstage);
+    const size_t b = step_smem_bytes<double, D, kCarryDoc>(pmax, nstage);
+    return a > b ? a : b;
+  }
+  return step_smem_bytes<float, D, kCarryNone>(pmax, nstage);
+}
+
 size_t update_smem_bytes(int d, fv_precision prec, int pmax, int nstage) {
-  const int es = prec == FV_FP64 ? 8 : 4;
-  return d == 1   ? step_smem_bytes<1>(es, pmax, nstage)
-         : d == 2 ? step_smem_bytes<2>(es, pmax, nstage)
-                  : step_smem_bytes<3>(es, pmax, nstage);
+  return d == 1   ? smem_by_prec<1>(prec, pmax, nstage)
+         : d == 2 ? smem_by_prec<2>(prec, pmax, nstage)
+                  : smem_by_prec<3>(prec, pmax, nstage);
 }
 
 template <typename T>
