@@ -10,6 +10,7 @@
 // in flight).
 #include "fv_device.cuh"
 #include "fv_internal.h"
+#include "fv_ptx.cuh"
 
 namespace fv {
 
@@ -84,6 +85,8 @@ __global__ void __launch_bounds__(FV_NT) halo_kernel(HaloParams<T> a) {
   constexpr int S = D + 2;
   constexpr int VEC = 16 / sizeof(T);
   constexpr int NW = FV_NT / 32;
+  grid_dep_wait();
+  grid_dep_launch();
   const int h = a.halo;
   const int lane = threadIdx.x & 31;
   for (int64_t i = (int64_t)blockIdx.x * NW + (threadIdx.x >> 5); i < a.n;
@@ -226,6 +229,8 @@ __global__ void __launch_bounds__(FV_NT) halo_kernel_pipe(HaloParams<T> a) {
   constexpr int NF = 2 * D;
   constexpr int VEC = 16 / sizeof(T);
   constexpr int NW = FV_NT / 32;
+  grid_dep_wait();
+  grid_dep_launch();
   const int h = a.halo;
   const int lane = threadIdx.x & 31;
   const int64_t wstep = (int64_t)gridDim.x * NW;
@@ -320,10 +325,11 @@ static cudaError_t launch_halo_t(const fv_batch* h, const HaloLaunch& l, int gri
   a.pmax = h->max_patch_size;
   a.status = l.status;
   if constexpr (D == 3)
-    halo_kernel_pipe<T, D><<<grid, FV_NT, 0, h->stream>>>(a);
+    return launch_kernel(halo_kernel_pipe<T, D>, grid, FV_NT, 0, h->stream,
+                         starts_early(h, grid), a);
   else
-    halo_kernel<T, D><<<grid, FV_NT, 0, h->stream>>>(a);
-  return cudaGetLastError();
+    return launch_kernel(halo_kernel<T, D>, grid, FV_NT, 0, h->stream,
+                         starts_early(h, grid), a);
 }
 
 cudaError_t launch_halo(const fv_batch* h, const HaloLaunch& l, int grid) {

@@ -196,6 +196,8 @@ __global__ void __launch_bounds__(kMNT, march_blocks<P>()) march3d_kernel(StepPa
   const int64_t warp = ((int64_t)blockIdx.x * kMNT + threadIdx.x) >> 5;
   const int64_t stride = (((int64_t)gridDim.x * kMNT) >> 5) * kMPW;
 
+  grid_dep_wait();
+  grid_dep_launch();
   double dtv;
   if constexpr (STEP) {
     const double lam = order_value<float>(*a.lam_in);
@@ -511,8 +513,8 @@ cudaError_t launch_march3d_t(const fv_batch* h, const UpdateLaunch& l, int grid)
   a.prim_stride = l.prim_stride;
   cudaError_t e = march3d_smem_attr<P, STEP, LAM>();
   if (e != cudaSuccess) return e;
-  march3d_kernel<P, STEP, LAM><<<grid, kMNT, MGeom<P>::BYTES, h->stream>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(march3d_kernel<P, STEP, LAM>, grid, kMNT, MGeom<P>::BYTES, h->stream,
+                       starts_early(h, grid), a);
 }
 
 template <int P, bool STEP>

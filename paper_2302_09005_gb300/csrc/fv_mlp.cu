@@ -121,18 +121,12 @@ __device__ __forceinline__ void st_bf16x4(unsigned char* dst, const float4& v) {
 }
 // A training step is a chain of two small kernels.  Each is launched while
 // the one before it still runs (programmatic dependent launch): it lets the
-// next one start, prepares what does not depend on the others, and waits here
+// next one start, prepares what does not depend on the others, and waits
 // until all of them are complete and their writes visible.  A step of 32,768
 // samples (256 tiles, one per CTA) is bound by the latency of that chain, not
 // by a unit: 35.5 us, with the parameters loaded one after the other, each
 // partial gradient's sum four loads deep and the loss summed by one thread;
 // 16.9 us with all loads of a phase in flight and the launches overlapped.
-__device__ __forceinline__ void grid_dep_launch() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void grid_dep_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
 
 template <bool TRAIN>
 __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
@@ -537,24 +531,6 @@ int mlp_grid(const fv_mlp_trainer* t, int64_t batch) {
   return (int)(tiles < t->grid_max ? tiles : t->grid_max);
 }
 
-// Launches a kernel of the chain; `early`: it may start while the kernel
-// before it on the stream, one of the chain too, still runs.
-template <typename K, typename A>
-cudaError_t launch_chain(K kernel, int grid, int threads, size_t smem, cudaStream_t stream,
-                         bool early, const A& args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = early ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
-}
-
 cudaError_t launch_net(const fv_mlp_trainer* t, bool train, const float* params, const float* x,
                        const float* target, int64_t batch, float* y, int* grid_out,
                        bool early) {
@@ -570,7 +546,7 @@ cudaError_t launch_net(const fv_mlp_trainer* t, bool train, const float* params,
   a.status = t->status;
   const int grid = mlp_grid(t, batch);
   if (grid_out) *grid_out = grid;
-  return launch_chain(train ? fv::mlp_kernel<true> : fv::mlp_kernel<false>, grid, fv::kRows,
+  return fv::launch_kernel(train ? fv::mlp_kernel<true> : fv::mlp_kernel<false>, grid, fv::kRows,
                       fv::kSmemBytes, t->stream, early, a);
 }
 
@@ -592,7 +568,7 @@ cudaError_t launch_update(const fv_mlp_trainer* t, int nparts, int64_t batch, fl
   u.c1 = grad_out ? 1.f : 1.f - powf(u.b1, (float)step);
   u.c2 = grad_out ? 1.f : 1.f - powf(u.b2, (float)step);
   u.loss_out = loss;
-  return launch_chain(fv::mlp_update_kernel, (fv::kMlpParams + 31) / 32, 256, 0, t->stream, true,
+  return fv::launch_kernel(fv::mlp_update_kernel, (fv::kMlpParams + 31) / 32, 256, 0, t->stream, true,
                       u);
 }
 

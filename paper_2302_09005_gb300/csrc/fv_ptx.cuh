@@ -126,4 +126,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// Programmatic dependent launch.  grid_dep_launch: the next kernel on the
+// stream, if launched for it, may start once every CTA of this one has got
+// here.  grid_dep_wait: until every kernel this one was launched early after
+// is complete and its writes are visible (at once for an ordinary launch).
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace fv

@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(FV_NT) eig_kernel(EigParams<T> a) {
   constexpr int VEC = 16 / sizeof(T);
   constexpr int NW = FV_NT / 32;
   __shared__ unsigned long long red[NW];
+  grid_dep_wait();
+  grid_dep_launch();
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t step = (int64_t)gridDim.x * NW;
   unsigned long long warp_max = 0ull;  // over this warp's patches
@@ -201,13 +203,23 @@ __global__ void __launch_bounds__(FV_NT) eig_kernel(EigParams<T> a) {
 
 // Reduces the per-CTA maxima (bit patterns of type T), writes the global
 // maximum and dt = cfl dx / (d lambda_max).
+struct EigFinish {
+  const unsigned long long* partials;
+  int nparts;
+  double* global_out;
+  unsigned long long* lam_slot;
+  double* dt_slot;
+  double* dt_out;
+  double cfl, dx;
+};
 template <typename T, int D>
-__global__ void eig_finish_kernel(const unsigned long long* __restrict__ partials, int nparts,
-                                  double* global_out, unsigned long long* lam_slot,
-                                  double* dt_slot, double* dt_out, double cfl, double dx) {
+__global__ void eig_finish_kernel(EigFinish a) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ unsigned long long red[32];
   unsigned long long m = 0ull;
-  for (int j = threadIdx.x; j < nparts; j += blockDim.x) m = partials[j] > m ? partials[j] : m;
+  for (int j = threadIdx.x; j < a.nparts; j += blockDim.x)
+    m = a.partials[j] > m ? a.partials[j] : m;
   m = warp_max_u64(m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
@@ -215,11 +227,11 @@ __global__ void eig_finish_kernel(const unsigned long long* __restrict__ partial
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = red[w] > m ? red[w] : m;
     m = red[0] > m ? red[0] : m;
     const double lam = order_value<T>(m);
-    if (global_out) *global_out = lam;
-    *lam_slot = m;  // bits, read by the next time step
-    const double dt = (cfl * dx) / ((double)D * lam);
-    *dt_slot = dt;
-    if (dt_out) *dt_out = dt;
+    if (a.global_out) *a.global_out = lam;
+    *a.lam_slot = m;  // bits, read by the next time step
+    const double dt = (a.cfl * a.dx) / ((double)D * lam);
+    *a.dt_slot = dt;
+    if (a.dt_out) *a.dt_out = dt;
   }
 }
 
@@ -237,8 +249,7 @@ static cudaError_t launch_eig_t(const fv_batch* h, const EigLaunch& l, int grid)
   a.per_patch = l.per_patch;
   a.partials = l.partials;
   a.status = l.status;
-  eig_kernel<T, D><<<grid, FV_NT, 0, h->stream>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(eig_kernel<T, D>, grid, FV_NT, 0, h->stream, starts_early(h, grid), a);
 }
 
 cudaError_t launch_eig(const fv_batch* h, const EigLaunch& l, int grid) {
@@ -255,20 +266,16 @@ cudaError_t launch_eig(const fv_batch* h, const EigLaunch& l, int grid) {
 cudaError_t launch_eig_finish(const fv_batch* h, const unsigned long long* partials, int nparts,
                               double* global_out, unsigned long long* lam_slot, double* dt_slot,
                               double* dt_out, double cfl, double dx) {
-#define FV_EIG_FIN(T, D)                                                                    \
-  eig_finish_kernel<T, D><<<1, 256, 0, h->stream>>>(partials, nparts, global_out, lam_slot, \
-                                                    dt_slot, dt_out, cfl, dx)
-  if (h->prec == FV_FP64) {
-    if (h->d == 1) FV_EIG_FIN(double, 1);
-    else if (h->d == 2) FV_EIG_FIN(double, 2);
-    else FV_EIG_FIN(double, 3);
-  } else {
-    if (h->d == 1) FV_EIG_FIN(float, 1);
-    else if (h->d == 2) FV_EIG_FIN(float, 2);
-    else FV_EIG_FIN(float, 3);
-  }
+  const EigFinish a{partials, nparts, global_out, lam_slot, dt_slot, dt_out, cfl, dx};
+#define FV_EIG_FIN(T, D) launch_kernel(eig_finish_kernel<T, D>, 1, 256, 0, h->stream, true, a)
+  if (h->prec == FV_FP64)
+    return h->d == 1   ? FV_EIG_FIN(double, 1)
+           : h->d == 2 ? FV_EIG_FIN(double, 2)
+                       : FV_EIG_FIN(double, 3);
+  return h->d == 1   ? FV_EIG_FIN(float, 1)
+         : h->d == 2 ? FV_EIG_FIN(float, 2)
+                     : FV_EIG_FIN(float, 3);
 #undef FV_EIG_FIN
-  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -457,6 +464,8 @@ __global__ void __cluster_dims__(kSumCluster, 1, 1) __launch_bounds__(NT)
   // the first CTA's shared memory may be written once every CTA has started
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   double total = 0.0;  // of unknown comp over the slice so far
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t i = i0 + v;
   int pn = 0;  // the next patch's metadata, loaded one patch ahead
   int64_t offn = 0;
@@ -512,21 +521,27 @@ __global__ void __cluster_dims__(kSumCluster, 1, 1) __launch_bounds__(NT)
   }
 }
 
+struct SumsFinish {
+  const double* partials;
+  int nchunks;
+  double* totals;
+};
 template <int S>
-__global__ void __launch_bounds__(FV_NT) sums_finish_kernel(const double* __restrict__ partials,
-                                                            int nchunks, double* totals) {
+__global__ void __launch_bounds__(FV_NT) sums_finish_kernel(SumsFinish a) {
   __shared__ double sh[FV_NT * S];
+  grid_dep_wait();
+  grid_dep_launch();
   double acc[S];
 #pragma unroll
   for (int k = 0; k < S; ++k) acc[k] = 0.0;
-  for (int c = threadIdx.x; c < nchunks; c += FV_NT) {
+  for (int c = threadIdx.x; c < a.nchunks; c += FV_NT) {
 #pragma unroll
-    for (int k = 0; k < S; ++k) acc[k] = acc[k] + partials[(int64_t)c * S + k];
+    for (int k = 0; k < S; ++k) acc[k] = acc[k] + a.partials[(int64_t)c * S + k];
   }
   block_sum_fixed<S>(acc, sh);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < S; ++k) totals[k] = acc[k];
+    for (int k = 0; k < S; ++k) a.totals[k] = acc[k];
   }
 }
 
@@ -543,10 +558,9 @@ static cudaError_t launch_sums_t(const fv_batch* h, const SumLaunch& l, int nchu
   a.status = l.status;
   a.per_patch = l.per_patch;
   if (nchunks <= kSumFewChunks)
-    sums_kernel<T, D, 512><<<nchunks * kSumCluster, 512, 0, h->stream>>>(a);
-  else
-    sums_kernel<T, D, 128><<<nchunks * kSumCluster, 128, 0, h->stream>>>(a);
-  return cudaGetLastError();
+    return launch_kernel(sums_kernel<T, D, 512>, nchunks * kSumCluster, 512, 0, h->stream,
+                         starts_early(h, nchunks * kSumCluster), a);
+  return launch_kernel(sums_kernel<T, D, 128>, nchunks * kSumCluster, 128, 0, h->stream, false, a);
 }
 
 cudaError_t launch_sums(const fv_batch* h, const SumLaunch& l, int nchunks) {
@@ -562,21 +576,24 @@ cudaError_t launch_sums(const fv_batch* h, const SumLaunch& l, int nchunks) {
 
 cudaError_t launch_sums_finish(const fv_batch* h, const double* partials, int nchunks,
                                double* totals) {
-  if (h->d == 1) sums_finish_kernel<3><<<1, FV_NT, 0, h->stream>>>(partials, nchunks, totals);
-  else if (h->d == 2) sums_finish_kernel<4><<<1, FV_NT, 0, h->stream>>>(partials, nchunks, totals);
-  else sums_finish_kernel<5><<<1, FV_NT, 0, h->stream>>>(partials, nchunks, totals);
-  return cudaGetLastError();
+  const SumsFinish a{partials, nchunks, totals};
+  if (h->d == 1) return launch_kernel(sums_finish_kernel<3>, 1, FV_NT, 0, h->stream, true, a);
+  if (h->d == 2) return launch_kernel(sums_finish_kernel<4>, 1, FV_NT, 0, h->stream, true, a);
+  return launch_kernel(sums_finish_kernel<5>, 1, FV_NT, 0, h->stream, true, a);
 }
 
 // ---------------------------------------------------------------------------
 // One 64-bit word set to zero on the stream (the wave-speed slot a time step
 // accumulates into, the work-queue counter), by a one-thread kernel.
 // ---------------------------------------------------------------------------
-__global__ void zero_word_kernel(unsigned long long* p) { *p = 0ull; }
+__global__ void zero_word_kernel(unsigned long long* p) {
+  grid_dep_wait();
+  grid_dep_launch();
+  *p = 0ull;
+}
 
 cudaError_t launch_zero_word(unsigned long long* p, cudaStream_t stream) {
-  zero_word_kernel<<<1, 1, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_kernel(zero_word_kernel, 1, 1, 0, stream, true, p);
 }
 
 // ---------------------------------------------------------------------------

@@ -196,6 +196,8 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
   const int64_t warp = (blockIdx.x * (int64_t)kRowsNT + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * kRowsNT) >> 5;
 
+  grid_dep_wait();
+  grid_dep_launch();
   double dtv;
   if constexpr (STEP) {
     const double lam = order_value<float>(*a.lam_in);
@@ -417,8 +419,8 @@ cudaError_t launch_rows2d_t(const fv_batch* h, const UpdateLaunch& l, int grid) 
   a.mzero = -0.0f;
   a.prim_out = static_cast<float*>(l.prim_out);
   a.prim_stride = l.prim_stride;
-  rows2d_kernel<P, STEP><<<grid, kRowsNT, RGeom<P>::BYTES, h->stream>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(rows2d_kernel<P, STEP>, grid, kRowsNT, RGeom<P>::BYTES, h->stream,
+                       starts_early(h, grid), a);
 }
 
 template <int P, bool STEP>

@@ -897,6 +897,8 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
     step_kernel(StepParams<T> a) {
   static_assert(CARRY == kCarryNone || (GATHER && FUSED), "the primitive carry is a time-step mode");
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  grid_dep_wait();
+  grid_dep_launch();
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
   unsigned long long* red = reinterpret_cast<unsigned long long*>(smem_raw + kRedOff);
   unsigned long long* run_max = reinterpret_cast<unsigned long long*>(smem_raw + kRunMaxOff);
@@ -1097,8 +1099,8 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
   const size_t smem = step_smem_bytes<T, D, CARRY>(l.pmax, a.nstage);
   cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
-  step_kernel<T, D, GATHER, FUSED, CARRY, NT><<<grid, NT, smem, h->stream>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(step_kernel<T, D, GATHER, FUSED, CARRY, NT>, grid, NT, smem, h->stream,
+                       starts_early(h, grid), a);
 }
 
 template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
