@@ -311,10 +311,10 @@ fv_status fv_time_step_prim(fv_batch* h, const void* in_with_halo, void* out,
  * fv_run_steps -- n_steps time steps from q0: fv_halo_fill and
  * fv_max_eigenvalue_reduce on q0, then fv_time_step_prim ping-ponging
  * between q0 and q1.  FP64 handles carry the primitives from step to step in
- * two buffers the handle allocates on first use (each n_patches * (2 d + 1) *
- * max_patch_size^d elements, rounded up to 16 bytes a patch, in a form of
- * their own; kept until fv_batch_destroy; growing them drops the cached
- * graphs); FP32 handles run without the carry (faster there).
+ * two buffers the handle allocates on first use (each n_patches *
+ * fv_prim_stride elements, a third more in 3D, in a form of their own; kept
+ * until fv_batch_destroy; growing them drops the cached graphs); FP32 handles
+ * run without the carry (faster there).
  * The result is in q0 if n_steps is even, else in q1.
  * use_graph != 0 captures the whole sequence into a CUDA graph the first
  * time a given set of arguments is seen, caches the instantiated graph in

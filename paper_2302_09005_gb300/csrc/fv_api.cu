@@ -155,7 +155,7 @@ fv_status fv_batch_create(fv_batch** out, int d, int s, const fv_options* o, voi
   // stages and CTAs per SM of the untuned launches (their CTA size follows the
   // patch size)
   const int nt = fv::default_nt(d, h->max_patch_size), ni = fv::nt_index(nt);
-  const int modes = opt.precision == FV_FP64 ? 4 : 3;
+  const int modes = opt.precision == FV_FP64 && d == 3 ? 4 : 3;
   for (int mode = fv::kModeUpdate; mode < modes && e == cudaSuccess; ++mode)
     e = fv::step_shape(h, mode, h->max_patch_size, nt, &h->nstage[mode][ni],
                        &h->blocks_per_sm[mode][ni]);
@@ -454,7 +454,7 @@ static fv_status time_step_impl(fv_batch* h, const void* in, void* out, const in
   l.prim_in = prim_in;
   l.prim_out = prim_out;
   l.prim_stride = fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, own);
-  l.prim_own = own;
+  l.prim_own = own && h->d == 3;
   e = fv::launch_scheduled(h, l);
   if (e != cudaSuccess) return cuda_err(h, e, "time step kernel");
   h->lam_cur = nxt;
@@ -473,22 +473,37 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
   // buffers, grown (never shrunk) before any capture; graphs that refer to
   // the old buffers are dropped when they move
   const bool carry = h->prec == FV_FP64 && n_steps > 1;
+  bool own = false;
   if (carry && n > 0) {
     const size_t es = h->prec == FV_FP64 ? 8 : 4;
-    const int64_t need = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, true);
-    if (need > h->prim_cap) {
+    const int64_t doc = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size);
+    const int64_t full = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, true);
+    // the library's own form, or, where memory does not allow it (3D: a third
+    // more), the documented one
+    if (full > h->prim_cap && !(h->prim_doc && doc <= h->prim_cap)) {
       cudaError_t e = cudaStreamSynchronize(h->stream);
       graph_cache_clear(h);
-      for (void*& pbuf : h->d_prim) {
-        if (pbuf) cudaFree(pbuf);
-        pbuf = nullptr;
-      }
       h->prim_cap = 0;
-      for (void*& pbuf : h->d_prim)
-        if (e == cudaSuccess) e = cudaMalloc(&pbuf, es * (size_t)need);
+      for (const int64_t need : {full, doc}) {
+        for (void*& pbuf : h->d_prim) {
+          if (pbuf) cudaFree(pbuf);
+          pbuf = nullptr;
+        }
+        if (e == cudaErrorMemoryAllocation) {
+          cudaGetLastError();
+          e = cudaSuccess;
+        }
+        for (void*& pbuf : h->d_prim)
+          if (e == cudaSuccess) e = cudaMalloc(&pbuf, es * (size_t)need);
+        if (e == cudaSuccess) {
+          h->prim_cap = need;
+          h->prim_doc = need < full;
+        }
+        if (e != cudaErrorMemoryAllocation) break;
+      }
       if (e != cudaSuccess) return cuda_err(h, e, "primitive buffers");
-      h->prim_cap = need;
     }
+    own = full <= h->prim_cap;
   }
   auto enqueue = [&]() -> fv_status {
     fv_status s = fv_halo_fill(h, q0, off, sizes, nbr, n);
@@ -501,7 +516,7 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
       const void* pin = (!carry || k == 0) ? nullptr : h->d_prim[(k - 1) & 1];
       void* pout = (carry && k + 1 < n_steps) ? h->d_prim[k & 1] : nullptr;
       s = time_step_impl(h, a, b, off, sizes, nbr, n, dx, cfl, nullptr, nullptr, pin, pout,
-                         carry);
+                         own);
       std::swap(a, b);
     }
     return s;

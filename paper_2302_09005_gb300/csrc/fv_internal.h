@@ -38,6 +38,7 @@ struct fv_batch {
   // primitive carry of fv_run_steps: two buffers of prim_cap elements
   void* d_prim[2] = {nullptr, nullptr};
   int64_t prim_cap = 0;
+  bool prim_doc = false;  // in the documented form: the library's own did not fit
   void* graph_cache = nullptr;               // captured multi-step graphs
   // schedule (fv_sched.cu): processing order sorted by size, size classes
   int sched = 0;                             // fv_schedule
@@ -92,7 +93,7 @@ struct UpdateLaunch {
   const void* prim_in = nullptr;  // time step: carried primitives of `in`, or null
   void* prim_out = nullptr;       // time step: primitives of `out`, or null
   int64_t prim_stride = 0;        // elements per patch of the primitive buffers
-  bool prim_own = false;          // FP64: both in fv_run_steps' own form
+  bool prim_own = false;          // 3D FP64: both in fv_run_steps' own form
   int uniform_p = 0;              // every patch of the launch has this size (0: unknown)
   unsigned long long* queue = nullptr;  // zeroed counter: CTAs pop positions (null: stride)
 };
@@ -111,10 +112,10 @@ inline int step_mode(const UpdateLaunch& l) {
 }
 
 // Elements per patch of a primitive buffer: (d + 3) p^d for p = pmax, rounded
-// up to 16 bytes; 2d + 1 components in fv_run_steps' own form (u, p and the
-// wave speeds |u_k| + c).
+// up to 16 bytes; 2d + 2 components in fv_run_steps' own form in 3D (u, p, E + p
+// and the wave speeds |u_k| + c).
 inline int64_t prim_stride_elems(int d, fv_precision prec, int pmax, bool own = false) {
-  int64_t c = own ? 2 * d + 1 : d + 3;
+  int64_t c = own && d == 3 ? 2 * d + 2 : d + 3;
   for (int k = 0; k < d; ++k) c *= pmax;
   const int64_t vec = prec == FV_FP64 ? 2 : 4;
   return (c + vec - 1) / vec * vec;

@@ -21,21 +21,27 @@
 //
 // Each CTA is persistent and walks its patches i = blockIdx.x + k*gridDim.x,
 // or pops them one at a time from a work queue (a zeroed device counter).
-// While it computes patch i, the TMA engine copies patch i+1 (and, carrying
-// primitives, their interior block) into the other of two shared-memory
-// stages (cp.async.bulk, completion on an mbarrier), and the halo cells of
-// patch i+1 that live elsewhere are gathered with cp.async.
+// With two shared-memory stages, the TMA engine copies patch i+1 (and,
+// carrying primitives, their interior block) into the other one while patch i
+// is computed (cp.async.bulk, completion on an mbarrier), and the halo cells of
+// patch i+1 that live elsewhere are gathered with cp.async; with one, patch
+// i+1 follows patch i and the other resident CTAs compute meanwhile (which
+// of the two: step_shape in fv_sched.cu).
 // Per patch:
 //   cells   (not when primitives are carried) every interior and face-halo
 //           cell converts to primitives once (Eq. 2); interior cells keep
 //           all of (u, p, c, E + p), halo cells the normal velocity, p, c,
-//           E + p.  The two groups start on warp boundaries;
+//           E + p (FP64: mostly |u_k| + c in the place of c, see kLamForm).
+//           The two groups start on warp boundaries;
 //   faces   every face flux G = f_L + f_R - a (Q_R - Q_L) = 2F (Eq. 4, 5) is
 //           computed exactly once, from the states and primitives of its two
 //           cells, and shared by both;
-//   update  every interior cell sums G_+ - G_- over x, then y, then z and
-//           writes Q - (dt / 2dx) sum (Eq. 3); a time step then converts the
-//           new state to primitives for the next CFL maximum (and the carry).
+//   update  every interior cell sums G_+ - G_- over x, y and z (FP32 in that
+//           order; FP64 with d >= 2 exactly, with one rounding, on the integer
+//           pipe: fv_fxsum.cuh) and writes Q - (dt / 2dx) sum (Eq. 3); a time
+//           step then converts the new state to primitives for the carry and
+//           the next CFL maximum (FP64 without a carry: only where FP32 bounds
+//           allow a new maximum).
 // Every floating-point operation is written out (fma or an explicitly
 // rounded add / multiply), so the compiler cannot contract differently in
 // different modes: the modes agree bitwise.  Maxima (per-patch a of
@@ -79,7 +85,7 @@ struct StepParams {
   int local_cfl;           // with dx_patch: dt_i = cfl dx_i / (d lambda_i) per patch
   const T* __restrict__ prim_in;  // carried primitives of `in` (primitive-carry mode)
   T* __restrict__ prim_out;       // primitives of `out` (time-step modes), or null
-  int prim_own;                   // FP64: prim_out in the library's own form (kCarryOwn)
+  int prim_own;                   // 3D FP64: prim_out in fv_run_steps' own form (kCarryOwn)
   int64_t prim_stride;            // elements per patch of prim_in / prim_out
   long long wait_limit = FV_WAIT_LIMIT;  // cycles of a wait for a patch's copy
   unsigned long long* queue = nullptr;    // zeroed counter of positions handed out, or null
@@ -98,37 +104,35 @@ __host__ __device__ inline int stage_elems(int p) {
 // a caller's carry in the documented form (u_1..u_D, p, c, E+p), or from
 // fv_run_steps' own buffers in the form the FP64 kernel works with.
 constexpr int kCarryNone = 0, kCarryDoc = 1, kCarryOwn = 2;
-// Interior primitives, components of p^D cells: in FP64 u_1..u_D, p and the
-// wave speeds |u_k| + c, k = 1..D, which every face of direction k takes from
-// its two cells (one addition a cell and direction where its two faces took
-// two each, and E + p is not needed at all); in FP32, and in the documented
-// carry, u_1..u_D, p, c, E+p.  With it the time step without the carry skips
-// the new state's primitives where they cannot raise the CFL maximum (see the
-// epilogue).  Measured with both: 20 steps of 200,000 uneven patches 95.3 ->
-// 88.7 ms, 9,177 6^3 patches' engine loop 667 -> 650 us, learned step 315 ->
-// 300 us, refined mesh 909 -> 879 us; the documented carry (energy flux without
-// E + p only) 6.25 -> 6.19 ms.
-template <typename T, int CARRY>
+// Interior primitives, components of p^D cells: u_1..u_D, p, c, E+p; or, in
+// FP64 where they are computed from the state or carried by fv_run_steps,
+// u_1..u_D, p, E+p and the wave speeds |u_k| + c, k = 1..D, which every face of
+// direction k takes from its two cells: one addition a cell and direction where
+// its two faces took two each.  3D, and 2D patches with a compile-time size (up
+// to 17; the sixth component of the largest 2D patches would not fit).  With it,
+// and the time step without a carry skipping the new state's primitives where
+// they cannot raise the CFL maximum (see the epilogue): 20 steps of 200,000
+// uneven patches 95.3 -> 90.2 ms, refined mesh 909 -> 894 us, engine loop of 9,177
+// 6^3 patches 667 -> 645 us, learned step 315 -> 310 us.
+template <typename T, int D, int CARRY, int P>
 constexpr bool kLamForm() {
-  return sizeof(T) == 8 && CARRY != kCarryDoc;
-}
-template <typename T, int D, int CARRY>
-__host__ __device__ constexpr int prim_comps() {
-  return kLamForm<T, CARRY>() ? 2 * D + 1 : D + 3;
+  return sizeof(T) == 8 &&
+         ((D == 3 && CARRY != kCarryDoc) || (D == 2 && CARRY == kCarryNone && P > 0));
 }
 template <typename T, int D, int CARRY>
 __host__ __device__ inline int iprim_elems(int p) {
-  return prim_comps<T, D, CARRY>() * ipow_d<D>(p);
+  if (kLamForm<T, D, CARRY, 0>()) return (2 * D + 2) * ipow_d<D>(p);
+  const int n = (D + 3) * ipow_d<D>(p);
+  if (!kLamForm<T, D, CARRY, 1>()) return n;
+  const int c = p < 17 ? p : 17;
+  const int m = (2 * D + 2) * ipow_d<D>(c);
+  return n > m ? n : m;
 }
-// Face-halo primitives: 2D faces x (u_normal, p, |u_normal| + c) in FP64
-// (c in the documented carry), (u_normal, p, c, E+p) in FP32 x p^(D-1).
-template <typename T>
-__host__ __device__ constexpr int halo_comps() {
-  return sizeof(T) == 8 ? 3 : 4;
-}
+// Face-halo primitives: 2D faces x (u_normal, p, c, E+p), or (u_normal, p, E+p,
+// |u_normal| + c) with the wave speeds, x p^(D-1).
 template <typename T, int D>
 __host__ __device__ inline int hprim_elems(int p) {
-  return 2 * D * halo_comps<T>() * (ipow_d<D>(p) / p);
+  return 2 * D * 4 * (ipow_d<D>(p) / p);
 }
 // face fluxes G: D directions x (D+2) unknowns x (p+1) p^(D-1) faces
 template <int D>
@@ -330,7 +334,7 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
     const int cs = g.cell_kt(k, m.ck, r);
     T* dst = s.box + cd * S;
     const T* src = a.in + m.off + (int64_t)cs * S;
-    T* pd = s.hp + f * halo_comps<T>() * ptr + r;
+    T* pd = s.hp + f * 4 * ptr + r;
     const T* ps = nullptr;
     if constexpr (CARRY != kCarryNone)
       ps = a.prim_in + (int64_t)m.pidx * a.prim_stride + g.icell_kt(k, m.ck - 1, r);
@@ -350,8 +354,8 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
     }
     if constexpr (CARRY != kCarryNone) {
       cp_async_elem(pd + ptr, ps + D * g.nint());
-      cp_async_elem(pd + 2 * ptr, ps + (D + 1 + (kLamForm<T, CARRY>() ? k : 0)) * g.nint());
-      if constexpr (halo_comps<T>() == 4) cp_async_elem(pd + 3 * ptr, ps + (D + 2) * g.nint());
+      cp_async_elem(pd + 2 * ptr, ps + (D + 1) * g.nint());
+      cp_async_elem(pd + 3 * ptr, ps + (D + 2 + (kLamForm<T, D, CARRY, P>() ? k : 0)) * g.nint());
     }
   };
   if constexpr (kGatherSlots<D, P, NT>()) {
@@ -563,9 +567,10 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
         for (int m = 0; m < D; ++m) ip[m * nint + t] = w.u[m];
         ip[D * nint + t] = w.p;
-        if constexpr (kLamForm<T, CARRY>()) {
+        if constexpr (kLamForm<T, D, CARRY, P>()) {
+          ip[(D + 1) * nint + t] = w.ep;
 #pragma unroll
-          for (int m = 0; m < D; ++m) ip[(D + 1 + m) * nint + t] = ar.add(abs_t(w.u[m]), w.c);
+          for (int m = 0; m < D; ++m) ip[(D + 2 + m) * nint + t] = ar.add(abs_t(w.u[m]), w.c);
         } else {
           ip[(D + 1) * nint + t] = w.c;
           ip[(D + 2) * nint + t] = w.ep;
@@ -583,11 +588,12 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
         T uk = w.u[0];
 #pragma unroll
         for (int m = 1; m < D; ++m) uk = (k == m) ? w.u[m] : uk;
-        T* h = hp + f * halo_comps<T>() * ptr + r;
+        T* h = hp + f * 4 * ptr + r;
         h[0] = uk;
         h[ptr] = w.p;
-        if constexpr (kLamForm<T, CARRY>()) {
-          h[2 * ptr] = ar.add(abs_t(uk), w.c);
+        if constexpr (kLamForm<T, D, CARRY, P>()) {
+          h[2 * ptr] = w.ep;
+          h[3 * ptr] = ar.add(abs_t(uk), w.c);
         } else {
           h[2 * ptr] = w.c;
           h[3 * ptr] = w.ep;
@@ -602,8 +608,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
   // Cell b (halo-inclusive, 0..p+1) along k at transverse index tr: its state
   // and the primitives of direction k (face-halo block at the patch
   // boundary, interior block inside).
-  // FP64: c is the wave speed |u| + c (the sound speed in the documented
-  // carry), e unused.
+  // With the wave speeds carried, c is |u| + c of the direction.
   struct CellK {
     T q[S];
     T u, pr, c, e;
@@ -617,15 +622,18 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     for (int v = 0; v < S; ++v) x.q[v] = st[cid * S + v];
     const bool h0 = lo && b == 0, h1 = hi && b == p + 1;
     const int ic = g.icell_kt(k, h0 ? 0 : (h1 ? p - 1 : b - 1), tr);
-    constexpr int HC = halo_comps<T>();
-    const T* h = hp + ((2 * k + (h1 ? 1 : 0)) * HC) * ptr + tr;
+    // after p: c, E + p; or E + p and, k + 1 components on (a halo cell: the
+    // next), the wave speed of direction k
+    constexpr bool LF = kLamForm<T, D, CARRY, P>();
+    const T* h = hp + (8 * k + (h1 ? 4 : 0)) * ptr + tr;
     const T* pu = (h0 || h1) ? h : ip + k * nint + ic;
     const T* pp_ = (h0 || h1) ? h + ptr : ip + D * nint + ic;
-    const int sp = (h0 || h1) ? ptr : nint * (kLamForm<T, CARRY>() ? k + 1 : 1);
+    const int sp = (h0 || h1) ? ptr : nint;
+    const int sw = (h0 || h1) ? 2 * ptr : (LF ? 2 + k : 2) * nint;
     x.u = pu[0];
     x.pr = pp_[0];
-    x.c = pp_[sp];
-    if constexpr (HC == 4) x.e = pp_[2 * sp];
+    x.c = pp_[LF ? sw : sp];
+    x.e = pp_[LF ? sp : sw];
   };
   // The flux of face j (k) between cells L and R, stored into G.
   auto flux = [&](const int k, const int j, const CellK& L, const CellK& R,
@@ -635,7 +643,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     const T* qL = L.q;
     const T* qR = R.q;
     // a = max(|u_k| + c) over the two cells (Eq. 5)
-    const T am = kLamForm<T, CARRY>()
+    const T am = kLamForm<T, D, CARRY, P>()
                      ? max_by_bits(cL, cR)
                      : max_by_bits(ar.add(abs_t(uL), cL), ar.add(abs_t(uR), cR));
     const unsigned long long ab = order_bits(am);
@@ -646,9 +654,9 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     // f + a Q folds to Q (u_k + a) (+ p): with s_L = u_L + a, s_R = u_R - a,
     //   G_rho = rho_L s_L + rho_R s_R,
     //   G_m   = j_mL s_L + j_mR s_R + (p_L + p_R) [m = k],
-    //   G_E   = E_L s_L + E_R s_R + p_L u_L + p_R u_R                     (FP64)
-    //         = (E + p)_L u_L + (E + p)_R u_R + a (E_L - E_R)             (FP32),
-    // four operations either way.
+    //   G_E   = (E + p)_L u_L + (E + p)_R u_R + a (E_L - E_R).
+    // (G_E as E_L s_L + E_R s_R + p_L u_L + p_R u_R costs the same and would spare
+    // E + p, but its terms are larger than their sum: it rounds worse.)
     const T sL = ar.add(uL, am), sR = ar.sub(uR, am);
     const T ps = ar.add(pL, pR);
     T gs[S];
@@ -656,10 +664,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
     for (int m = 0; m < D; ++m)
       gs[1 + m] = fma(qL[1 + m], sL, fma(qR[1 + m], sR, (m == k) ? ps : T(-0.0)));
-    if constexpr (sizeof(T) == 8)
-      gs[D + 1] = fma(qL[D + 1], sL, fma(qR[D + 1], sR, fma(pL, uL, ar.mul(pR, uR))));
-    else
-      gs[D + 1] = fma(am, ar.sub(qL[D + 1], qR[D + 1]), fma(L.e, uL, ar.mul(R.e, uR)));
+    gs[D + 1] = fma(am, ar.sub(qL[D + 1], qR[D + 1]), fma(L.e, uL, ar.mul(R.e, uR)));
     T* Gk = G + k * S * nface;
 #pragma unroll
     for (int v = 0; v < S; ++v) {
@@ -835,9 +840,10 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
             for (int m = 0; m < D; ++m) po[m * nint] = w.u[m];
             po[D * nint] = w.p;
-            if (a.prim_own) {
+            if (D == 3 && a.prim_own) {
+              po[(D + 1) * nint] = w.ep;
 #pragma unroll
-              for (int m = 0; m < D; ++m) po[(D + 1 + m) * nint] = lam[m];
+              for (int m = 0; m < D; ++m) po[(D + 2 + m) * nint] = lam[m];
             } else {
               po[(D + 1) * nint] = w.c;
               po[(D + 2) * nint] = w.ep;
@@ -1136,8 +1142,8 @@ cudaError_t launch_step_nt(const fv_batch* h, const UpdateLaunch& l, int grid) {
   const int mode = step_mode(l);
   if (mode == kModePrim) return launch_by_d<T, NT, true, true, kCarryDoc>(h, l, grid);
   if (mode == kModeStep) return launch_by_d<T, NT, true, true, kCarryNone>(h, l, grid);
-  if (mode == kModeOwn) {  // fv_run_steps carries in FP64 only
-    if constexpr (sizeof(T) == 8) return launch_by_d<T, NT, true, true, kCarryOwn>(h, l, grid);
+  if (mode == kModeOwn) {  // 3D FP64 (see UpdateLaunch::prim_own)
+    if constexpr (sizeof(T) == 8) return launch_step_t<T, 3, true, true, kCarryOwn, NT>(h, l, grid);
     return cudaErrorInvalidConfiguration;
   }
   return launch_by_d<T, NT, false, false, kCarryNone>(h, l, grid);
@@ -1149,7 +1155,7 @@ cudaError_t occupancy_nt(int d, int mode, int pmax, int nstage, int* bps) {
   if (mode == kModeStep) return occupancy_by_d<T, NT, true, true, kCarryNone>(d, pmax, nstage, bps);
   if (mode == kModeOwn) {
     if constexpr (sizeof(T) == 8)
-      return occupancy_by_d<T, NT, true, true, kCarryOwn>(d, pmax, nstage, bps);
+      return occupancy_t<T, 3, true, true, kCarryOwn, NT>(pmax, nstage, bps);
     return cudaErrorInvalidConfiguration;
   }
   return occupancy_by_d<T, NT, false, false, kCarryNone>(d, pmax, nstage, bps);
