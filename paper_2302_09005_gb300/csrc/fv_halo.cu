@@ -326,10 +326,10 @@ static cudaError_t launch_halo_t(const fv_batch* h, const HaloLaunch& l, int gri
   a.status = l.status;
   if constexpr (D == 3)
     return launch_kernel(halo_kernel_pipe<T, D>, grid, FV_NT, 0, h->stream,
-                         starts_early(h, grid), a);
+                         starts_early(h, grid, FV_NT), a);
   else
     return launch_kernel(halo_kernel<T, D>, grid, FV_NT, 0, h->stream,
-                         starts_early(h, grid), a);
+                         starts_early(h, grid, FV_NT), a);
 }
 
 cudaError_t launch_halo(const fv_batch* h, const HaloLaunch& l, int grid) {

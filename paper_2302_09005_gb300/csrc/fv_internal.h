@@ -257,12 +257,15 @@ cudaError_t launch_selftest_math(const double* x, double* out, int64_t n, int wh
 // of the stream holds for everything that is visible; what overlaps is the
 // launch itself.
 //
-// starts_early: the rule for the patch kernels.  A grid that leaves the GPU
-// mostly empty is bound by launch latency (an update of 64 3x3 patches, FP64:
-// 8.19 -> 5.78 us per call); a larger one would find its SMs unevenly occupied
-// by the kernel it follows and keep that unevenness (20 steps of 670,761 5x5
-// patches, FP32: 4.83 -> 4.89 ms).
-inline bool starts_early(const fv_batch* h, int grid) { return grid <= 2 * h->num_sms; }
+// starts_early: the rule for the patch kernels, at most 256 threads per SM.  A
+// launch that leaves the GPU mostly empty is bound by launch latency (an update
+// of 64 3x3 patches, FP64: 8.19 -> 5.78 us per call); a larger one would find
+// its SMs unevenly occupied by the kernel it follows and keep that unevenness
+// (20 steps of 670,761 5x5 patches, FP32: 4.83 -> 4.89 ms; 300 updates of 8^3,
+// 256 threads each, FP32: 14.4 -> 17.1 us).
+inline bool starts_early(const fv_batch* h, int grid, int threads) {
+  return (int64_t)grid * threads <= (int64_t)h->num_sms * 256;
+}
 
 template <typename K, typename A>
 inline cudaError_t launch_kernel(K kernel, int grid, int threads, size_t smem, cudaStream_t stream,

@@ -514,7 +514,7 @@ cudaError_t launch_march3d_t(const fv_batch* h, const UpdateLaunch& l, int grid)
   cudaError_t e = march3d_smem_attr<P, STEP, LAM>();
   if (e != cudaSuccess) return e;
   return launch_kernel(march3d_kernel<P, STEP, LAM>, grid, kMNT, MGeom<P>::BYTES, h->stream,
-                       starts_early(h, grid), a);
+                       starts_early(h, grid, kMNT), a);
 }
 
 template <int P, bool STEP>

@@ -249,7 +249,7 @@ static cudaError_t launch_eig_t(const fv_batch* h, const EigLaunch& l, int grid)
   a.per_patch = l.per_patch;
   a.partials = l.partials;
   a.status = l.status;
-  return launch_kernel(eig_kernel<T, D>, grid, FV_NT, 0, h->stream, starts_early(h, grid), a);
+  return launch_kernel(eig_kernel<T, D>, grid, FV_NT, 0, h->stream, starts_early(h, grid, FV_NT), a);
 }
 
 cudaError_t launch_eig(const fv_batch* h, const EigLaunch& l, int grid) {
@@ -559,7 +559,7 @@ static cudaError_t launch_sums_t(const fv_batch* h, const SumLaunch& l, int nchu
   a.per_patch = l.per_patch;
   if (nchunks <= kSumFewChunks)
     return launch_kernel(sums_kernel<T, D, 512>, nchunks * kSumCluster, 512, 0, h->stream,
-                         starts_early(h, nchunks * kSumCluster), a);
+                         starts_early(h, nchunks * kSumCluster, 512), a);
   return launch_kernel(sums_kernel<T, D, 128>, nchunks * kSumCluster, 128, 0, h->stream, false, a);
 }
 

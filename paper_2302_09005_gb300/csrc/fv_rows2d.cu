@@ -420,7 +420,7 @@ cudaError_t launch_rows2d_t(const fv_batch* h, const UpdateLaunch& l, int grid) 
   a.prim_out = static_cast<float*>(l.prim_out);
   a.prim_stride = l.prim_stride;
   return launch_kernel(rows2d_kernel<P, STEP>, grid, kRowsNT, RGeom<P>::BYTES, h->stream,
-                       starts_early(h, grid), a);
+                       starts_early(h, grid, kRowsNT), a);
 }
 
 template <int P, bool STEP>

@@ -1106,7 +1106,7 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
   cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
   return launch_kernel(step_kernel<T, D, GATHER, FUSED, CARRY, NT>, grid, NT, smem, h->stream,
-                       starts_early(h, grid), a);
+                       starts_early(h, grid, NT), a);
 }
 
 template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>

@@ -126,3 +126,37 @@ def test_captured_time_steps_replay(fv, prec, steps):
         b.close()
     assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
     assert res[0][2] == res[1][2]
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_event_waits_hold(fv, prec):
+    """A launch after a wait on another stream's event sees what that stream
+    wrote, although the kernel before it on its own stream lets it start early:
+    the other stream is kept busy, then changes the input."""
+    torch = fvtest.torch_cuda()
+    d, p, n = 2, 4, 20
+    q, off, sz = fvtest.random_batch(n, p, d, 7, np.float32 if prec else np.float64)
+    toff, tsz = fvtest.to_dev(off), fvtest.to_dev(sz)
+    old, new = fvtest.to_dev(q), fvtest.to_dev(q) * 1.25
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    x, y, ref = old.clone(), torch.zeros_like(old), torch.zeros_like(old)
+    torch.cuda.synchronize()
+    b = fv.Batch(d, precision=prec, max_patch_size=p, stream=one)
+    b.update(new, ref, toff, tsz, 0.01, 1e-3)
+    torch.cuda.synchronize()
+    for _ in range(5):
+        x.copy_(old)
+        y.zero_()
+        torch.cuda.synchronize()
+        ev = torch.cuda.Event()
+        with torch.cuda.stream(two):
+            torch.cuda._sleep(2_000_000)  # about a millisecond
+            x.copy_(new)
+            ev.record(two)
+        b.update(old, y, toff, tsz, 0.01, 1e-3)  # its end lets the next one start
+        one.wait_event(ev)
+        b.update(x, y, toff, tsz, 0.01, 1e-3)
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref)
+    assert b.status() == fv.FV_OK
+    b.close()
