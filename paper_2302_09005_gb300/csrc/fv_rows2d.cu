@@ -43,27 +43,23 @@ constexpr int kRowsGroup = 8;    // lanes per patch
 constexpr int kRowsPerWarp = 4;  // patches per warp and iteration
 
 __device__ __forceinline__ unsigned umax_u(unsigned a, unsigned b) { return a > b ? a : b; }
-// |u| + c of a cell as its IEEE bits (>= 0 or NaN, so unsigned maxima order
-// them like the values)
-__device__ __forceinline__ unsigned wave_bits_f(float u, float c) {
-  return __float_as_uint(add_rn(fabsf(u), c));
-}
 constexpr unsigned kMag = 0x7FFFFFFFu;
 // positivity of rho and p accumulated as max(bits - 1): 0 < x < inf <=>
 // bits(x) - 1 < 0x7F7FFFFF
 constexpr unsigned kBad = 0x7F7FFFFFu;
 constexpr unsigned kSignR = 0x80000000u;  // the sign bit: a wall's mirrored momentum
 
-// State and primitives of one cell: rho, j_x, j_y, E; u_x, u_y, p, c, E + p.
+// State and primitives of one cell: rho, j_x, j_y, E; u_x, u_y, p, E + p, and
+// the wave speeds |u_k| + c (>= 0 or NaN, so unsigned maxima of their bits
+// order them like the values).
 struct RCell {
   float q[4];
-  float u[2], p, c, e;
+  float u[2], p, e, w[2];
 };
 
 // Primitives (Eq. 2) with the operations, in order, of primitives<float, 2>()
-// of the general kernel; `need` keeps non-cells out of the positivity check.
-__device__ __forceinline__ void rprims(RCell& x, float gm1, float gamma, bool need,
-                                       unsigned& chk) {
+// of the general kernel; returns c.
+__device__ __forceinline__ float rprims(RCell& x, float gm1, float gamma, unsigned& chk) {
   const float inv = recip(x.q[0]);
   x.u[0] = mul_rn(x.q[1], inv);
   x.u[1] = mul_rn(x.q[2], inv);
@@ -71,10 +67,11 @@ __device__ __forceinline__ void rprims(RCell& x, float gm1, float gamma, bool ne
   jj = fmaf(x.q[2], x.u[1], jj);
   x.p = mul_rn(gm1, fmaf(-0.5f, jj, x.q[3]));
   x.e = add_rn(x.q[3], x.p);
-  x.c = sqrt_t(mul_rn(mul_rn(gamma, x.p), inv));
-  const unsigned m = need ? ~0u : 0u;
-  chk = umax_u(chk, (__float_as_uint(x.q[0]) - 1u) & m);
-  chk = umax_u(chk, (__float_as_uint(x.p) - 1u) & m);
+  const float c = sqrt_t(mul_rn(mul_rn(gamma, x.p), inv));
+  x.w[0] = add_rn(fabsf(x.u[0]), c);
+  x.w[1] = add_rn(fabsf(x.u[1]), c);
+  chk = umax_u(chk, umax_u(__float_as_uint(x.q[0]) - 1u, __float_as_uint(x.p) - 1u));
+  return c;
 }
 
 // G = 2F of one face along k (Eq. 4, 5) in the general kernel's operation
@@ -82,7 +79,7 @@ __device__ __forceinline__ void rprims(RCell& x, float gm1, float gamma, bool ne
 template <int K>
 __device__ __forceinline__ unsigned rflux(const RCell& L, const RCell& R, float (&g)[4]) {
   constexpr int N = 1 + K, T = 2 - K;  // normal and transverse momentum
-  const unsigned ab = umax_u(wave_bits_f(L.u[K], L.c), wave_bits_f(R.u[K], R.c));
+  const unsigned ab = umax_u(__float_as_uint(L.w[K]), __float_as_uint(R.w[K]));
   const float am = __uint_as_float(ab);
   const float sL = add_rn(L.u[K], am), sR = sub_rn(R.u[K], am), ps = add_rn(L.p, R.p);
   g[0] = fmaf(L.q[0], sL, mul_rn(R.q[0], sR));
@@ -91,7 +88,6 @@ __device__ __forceinline__ unsigned rflux(const RCell& L, const RCell& R, float 
   g[3] = fmaf(am, sub_rn(L.q[3], R.q[3]), fmaf(L.e, L.u[K], mul_rn(R.e, R.u[K])));
   return ab;
 }
-
 
 // Shared-memory staging (floats) of patch size P, per group and stage: the
 // rows 1 .. P of the own box with their x-halo cells (A, one contiguous
@@ -184,7 +180,14 @@ constexpr int rows_blocks() {
   return P <= 5 ? FV_ROWS2D_MINBLOCKS : 12;
 }
 
-template <int P, bool STEP>
+// Bound by instruction issue and latency at 16 warps per SM.  Every wave speed
+// |u_k| + c is computed once per cell (not at both faces; the y ones travel with
+// the shuffles in the place of c), the positivity check needs no masks (what is
+// not loaded holds a benign state) and the faces' maxima are compiled only into
+// the launches that ask for them: 20 steps of 670,761 patches of 5x5 4.82 -> 4.77
+// ms.  (Two cells at a time in packed pairs took out more instructions, 237 ->
+// 217 per patch, but not more time: 4.73 ms, and lost on the 3D sweep.)
+template <int P, bool STEP, bool LAM>
 __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepParams<float> a) {
   constexpr int S = 4, NE = P + 2;
   static_assert(NE <= kRowsGroup, "a patch's rows fit one lane group");
@@ -275,9 +278,9 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
         for (int x = 1; x <= P; ++x) st_cell(c[x], row + (x - 1) * S, 0u, nm2);
       }
     }
+    // (cells not loaded hold the benign state, which passes the check)
 #pragma unroll
-    for (int x = 0; x < NE; ++x)
-      rprims(c[x], gm1, gam, on && (inner || (x >= 1 && x <= P)), chk);
+    for (int x = 0; x < NE; ++x) rprims(c[x], gm1, gam, chk);
 
     unsigned lmax = 0u;
     // ---- x faces of an interior row: flux differences of its cells -------
@@ -285,12 +288,12 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
     {
       float gprev[S];
       const unsigned ab = rflux<0>(c[0], c[1], gprev);
-      lmax = umax_u(lmax, ab & (inner ? kMag : 0u));
+      if constexpr (LAM) lmax = ab;
 #pragma unroll
       for (int x = 1; x <= P; ++x) {
         float g[S];
         const unsigned abx = rflux<0>(c[x], c[x + 1], g);
-        lmax = umax_u(lmax, abx & (inner ? kMag : 0u));
+        if constexpr (LAM) lmax = umax_u(lmax, abx);
 #pragma unroll
         for (int v = 0; v < S; ++v) {
           dg[x - 1][v] = sub_rn(g[v], gprev[v]);
@@ -299,6 +302,8 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
       }
     }
 
+    if (!inner) lmax = 0u;
+    unsigned ymax = 0u;
     // ---- y faces: rows r | r + 1 of every interior column ----------------
     float gy[P][S];
 #pragma unroll
@@ -308,15 +313,17 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
       for (int v = 0; v < S; ++v) up.q[v] = shfl_dn(c[x].q[v]);
       up.u[1] = shfl_dn(c[x].u[1]);
       up.p = shfl_dn(c[x].p);
-      up.c = shfl_dn(c[x].c);
+      up.w[1] = shfl_dn(c[x].w[1]);
       up.e = shfl_dn(c[x].e);
       float g[S];
       const unsigned ab = rflux<1>(c[x], up, g);
-      lmax = umax_u(lmax, ab & ((act && yface) ? kMag : 0u));
+      if constexpr (LAM) ymax = umax_u(ymax, ab);
 #pragma unroll
       for (int v = 0; v < S; ++v) gy[x - 1][v] = g[v];
     }
-    if (a.lam_patch != nullptr) {  // the patch's maximum over its eight lanes
+    if constexpr (LAM) {  // the patch's maximum over its eight lanes
+      if (act && yface) lmax = umax_u(lmax, ymax);
+      lmax &= kMag;
       lmax = umax_u(lmax, __shfl_xor_sync(0xFFFFFFFFu, lmax, 4));
       lmax = umax_u(lmax, __shfl_xor_sync(0xFFFFFFFFu, lmax, 2));
       lmax = umax_u(lmax, __shfl_xor_sync(0xFFFFFFFFu, lmax, 1));
@@ -341,16 +348,15 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
           RCell w;
 #pragma unroll
           for (int v = 0; v < S; ++v) w.q[v] = qn[v];
-          rprims(w, gm1, gam, true, chk);
-#pragma unroll
-          for (int k = 0; k < 2; ++k) lam_next = umax_u(lam_next, wave_bits_f(w.u[k], w.c) & kMag);
+          const float cn = rprims(w, gm1, gam, chk);
+          lam_next = umax_u(lam_next, umax_u(__float_as_uint(w.w[0]), __float_as_uint(w.w[1])));
           if (a.prim_out != nullptr) {
             constexpr int NI = P * P;
             float* po = a.prim_out + pid * a.prim_stride + (x - 1) + P * (r - 1);
             po[0] = w.u[0];
             po[NI] = w.u[1];
             po[2 * NI] = w.p;
-            po[3 * NI] = w.c;
+            po[3 * NI] = cn;
             po[4 * NI] = w.e;
           }
         }
@@ -383,12 +389,12 @@ __global__ void __launch_bounds__(kRowsNT, rows_blocks<P>()) rows2d_kernel(StepP
   cp_async_wait_all();
   if (__any_sync(0xFFFFFFFFu, chk >= kBad) && lane == 0) atomicOr(a.status, ST_NONPHYSICAL);
   if constexpr (STEP) {
-    const unsigned long long m = warp_max_u64((unsigned long long)lam_next);
+    const unsigned long long m = warp_max_u64((unsigned long long)(lam_next & kMag));
     if (lane == 0 && m != 0ull) atomicMax(a.lam_next, m);
   }
 }
 
-template <int P, bool STEP>
+template <int P, bool STEP, bool LAM>
 cudaError_t launch_rows2d_t(const fv_batch* h, const UpdateLaunch& l, int grid) {
   StepParams<float> a{};
   a.in = static_cast<const float*>(l.in);
@@ -419,13 +425,13 @@ cudaError_t launch_rows2d_t(const fv_batch* h, const UpdateLaunch& l, int grid) 
   a.mzero = -0.0f;
   a.prim_out = static_cast<float*>(l.prim_out);
   a.prim_stride = l.prim_stride;
-  return launch_kernel(rows2d_kernel<P, STEP>, grid, kRowsNT, RGeom<P>::BYTES, h->stream,
+  return launch_kernel(rows2d_kernel<P, STEP, LAM>, grid, kRowsNT, RGeom<P>::BYTES, h->stream,
                        starts_early(h, grid, kRowsNT), a);
 }
 
 template <int P, bool STEP>
 cudaError_t occupancy_rows2d_t(int* bps) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, rows2d_kernel<P, STEP>, kRowsNT,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, rows2d_kernel<P, STEP, true>, kRowsNT,
                                                        RGeom<P>::BYTES);
 }
 
@@ -445,8 +451,12 @@ int rows2d_patches_per_cta() { return (kRowsNT / 32) * kRowsPerWarp; }
 
 template <int P>
 static cudaError_t launch_rows2d_p(const fv_batch* h, const UpdateLaunch& l, int grid) {
-  return step_mode(l) == kModeStep ? launch_rows2d_t<P, true>(h, l, grid)
-                                   : launch_rows2d_t<P, false>(h, l, grid);
+  const bool step = step_mode(l) == kModeStep, lam = l.lam_patch != nullptr;
+  if (step)
+    return lam ? launch_rows2d_t<P, true, true>(h, l, grid)
+               : launch_rows2d_t<P, true, false>(h, l, grid);
+  return lam ? launch_rows2d_t<P, false, true>(h, l, grid)
+             : launch_rows2d_t<P, false, false>(h, l, grid);
 }
 
 cudaError_t launch_rows2d(const fv_batch* h, const UpdateLaunch& l, int grid) {
