@@ -12,8 +12,10 @@
 // Weights, X, H1, H2, dY, dZ2 and dZ1 enter the products rounded to BF16; the
 // accumulators, Z, the master parameters, gradients and Adam moments are FP32.
 //
-// One CTA of 128 threads walks tiles of 128 samples (thread t owns sample t
-// of the tile, which is TMEM lane t of every accumulator).  Per tile, one
+// One CTA of 256 threads walks tiles of 128 samples (threads t and t + 128 own
+// sample t of the tile, which is TMEM lane t of every accumulator, and half
+// of its 64 hidden units each: a row pass is a chain of loads, activations and
+// stores whose latency halves with its length).  Per tile, one
 // elected thread issues the chain of products, and after each the threads
 // read their rows back, apply the bias and activation and write the next
 // operand:
@@ -53,6 +55,7 @@ namespace {
 //   PA: [dZ2 (64) | dZ1 (64)]
 //   PB: [H2 (64) | ones row, zeros]
 constexpr int kRows = 128;      // samples per tile: the MMA's M
+constexpr int kNT = 256;        // threads per CTA: two per sample
 constexpr int kGroup = 2048;    // bytes per 8 samples in a paired buffer
 constexpr int kPC = 0, kPA = 32768, kPB = 65536;
 constexpr int kXoff = 1024, kOnesC = 1280, kDYoff = 1536, kOnesB = 1024;
@@ -126,26 +129,28 @@ __device__ __forceinline__ void st_bf16x4(unsigned char* dst, const float4& v) {
 // samples (256 tiles, one per CTA) is bound by the latency of that chain, not
 // by a unit: 35.5 us, with the parameters loaded one after the other, each
 // partial gradient's sum four loads deep and the loss summed by one thread;
-// 16.9 us with all loads of a phase in flight and the launches overlapped.
-
+// 17.0 us with all loads of a phase in flight and the launches overlapped, 16.1
+// with two threads per sample.
 template <bool TRAIN>
-__global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
+__global__ void __launch_bounds__(kNT, 2) mlp_kernel(MlpArgs a) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ alignas(8) uint64_t bar;
   __shared__ uint32_t tslot;
   __shared__ float red[kRows / 32];
   const int tid = threadIdx.x, warp = tid >> 5;
+  const int trow = tid & (kRows - 1), half = tid >> 7;  // the sample, the half of its units
+  const int c0 = 32 * half;                             // the half's first unit
   float* bias = reinterpret_cast<float*>(sm + kBias);
 
   if (TRAIN) {
     // the constant rows: ones at feature 80 of PC (B of GA) and at row 64 of
     // PB (A of GW3), zeros around them
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = tid; i < 16 * 16; i += kRows) {  // 16 groups x 16 chunks of 16 B
+    for (int i = tid; i < 16 * 16; i += kNT) {  // 16 groups x 16 chunks of 16 B
       const int g = i >> 4, c = i & 15;
       *reinterpret_cast<uint4*>(sm + kPC + g * kGroup + kOnesC + c * 16) = z;
     }
-    for (int i = tid; i < 16 * 64; i += kRows) {
+    for (int i = tid; i < 16 * 64; i += kNT) {
       const int g = i >> 6, c = i & 63;
       *reinterpret_cast<uint4*>(sm + kPB + g * kGroup + kOnesB + c * 16) = z;
     }
@@ -162,15 +167,15 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
   }
   if (warp == 0) tc_alloc(&tslot, kTmemCols);
   const int64_t ntiles = (a.rows + kRows - 1) / kRows;
-  float4 xv[4], tv = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 xv[2], tv = make_float4(0.f, 0.f, 0.f, 0.f);
   auto load_rows = [&](int64_t tile) {
-    const int64_t r = tile * kRows + tid;
+    const int64_t r = tile * kRows + trow;
     const bool ok = tile < ntiles && r < a.rows;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      xv[i] = ok ? __ldg(reinterpret_cast<const float4*>(a.x + r * 16) + i)
+    for (int i = 0; i < 2; ++i)
+      xv[i] = ok ? __ldg(reinterpret_cast<const float4*>(a.x + r * 16) + 2 * half + i)
                  : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (TRAIN) tv = ok ? __ldg(reinterpret_cast<const float4*>(a.t + r * 4))
+    if (TRAIN) tv = ok && half == 0 ? __ldg(reinterpret_cast<const float4*>(a.t + r * 4))
                        : make_float4(0.f, 0.f, 0.f, 0.f);
   };
   load_rows(blockIdx.x);  // the samples are no kernel's output
@@ -180,39 +185,28 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     // weights as BF16 K-major tiles, four of a row at a time, every load in
     // flight before the first store; biases
     const bool vec = ((uintptr_t)a.params & 15u) == 0;
-    float4 w1[2], w2[8], w3 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 w1, w2[4], w3 = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w2[i] = ld_par4(a.params + kOffW2 + 4 * (tid + i * kRows), vec);
+    for (int i = 0; i < 4; ++i) w2[i] = ld_par4(a.params + kOffW2 + 4 * (tid + i * kNT), vec);
+    w1 = ld_par4(a.params + kOffW1 + 4 * tid, vec);
+    if (tid < 64) w3 = ld_par4(a.params + kOffW3 + 4 * tid, vec);  // rows 4 .. 15 are zero
+    const int ib = tid < 64 ? kOffB1 + tid : tid < 128 ? kOffB2 + tid - 64 : kOffB3 + tid - 128;
+    const float bb = tid < 132 ? a.params[ib] : 0.f;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) w1[i] = ld_par4(a.params + kOffW1 + 4 * (tid + i * kRows), vec);
-    if (tid < 64) w3 = ld_par4(a.params + kOffW3 + 4 * tid, vec);
-    const float bb = a.params[tid < 64 ? kOffB1 + tid : kOffB2 + tid - 64];
-    const float b3 = tid < 4 ? a.params[kOffB3 + tid] : 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int e = 4 * (tid + i * kRows);
+    for (int i = 0; i < 4; ++i) {
+      const int e = 4 * (tid + i * kNT);
       st_bf16x4(sm + kW2 + kmajor(e >> 6, e & 63, 64), w2[i]);
     }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int e = 4 * (tid + i * kRows);
-      st_bf16x4(sm + kW1 + kmajor(e >> 4, e & 15, 16), w1[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {  // rows 4 .. 15 of W3 are zero
-      const int e = 4 * (tid + i * kRows);
-      st_bf16x4(sm + kW3 + kmajor(e >> 6, e & 63, 64),
-                e < 4 * 64 ? w3 : make_float4(0.f, 0.f, 0.f, 0.f));
-    }
-    bias[tid] = bb;
-    if (tid < 4) bias[128 + tid] = b3;
+    st_bf16x4(sm + kW1 + kmajor((4 * tid) >> 4, (4 * tid) & 15, 16), w1);
+    st_bf16x4(sm + kW3 + kmajor((4 * tid) >> 6, (4 * tid) & 63, 64), w3);
+    if (tid < 132) bias[tid] = bb;
   }
   fence_proxy_async_smem();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tm = tslot;
-  const uint32_t lane_base = tm + ((uint32_t)(warp * 32) << 16);  // this warp's lanes
+  const uint32_t lane_base = tm + ((uint32_t)((warp & 3) * 32) << 16);  // this warp's lanes
   const uint32_t tW = lane_base + kColW, tZ2 = lane_base + kColZ2;
   const uint32_t tG3 = lane_base + kColG3, tGA = lane_base + kColGA;
 
@@ -248,14 +242,12 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
   float loss = 0.f;
   bool first = true;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t row = tile * kRows + tid;
+    const int64_t row = tile * kRows + trow;
     const bool valid = row < a.rows;
     const float4 tcur = tv;
     {  // X -> PC
-      float v[16] = {xv[0].x, xv[0].y, xv[0].z, xv[0].w, xv[1].x, xv[1].y, xv[1].z, xv[1].w,
-                     xv[2].x, xv[2].y, xv[2].z, xv[2].w, xv[3].x, xv[3].y, xv[3].z, xv[3].w};
-      st_bf16x8(sm + kPC + prow(tid, kXoff, 0), v);
-      st_bf16x8(sm + kPC + prow(tid, kXoff, 1), v + 8);
+      float v[8] = {xv[0].x, xv[0].y, xv[0].z, xv[0].w, xv[1].x, xv[1].y, xv[1].z, xv[1].w};
+      st_bf16x8(sm + kPC + prow(trow, kXoff, half), v);
     }
     load_rows(tile + gridDim.x);  // the next tile's rows arrive during this one
     handoff();
@@ -264,13 +256,13 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     // ---- H1 = gelu(Z1 + b1) -> PC
     if (!failed) {
 #pragma unroll
-      for (int c = 0; c < 64; c += 16) {
+      for (int c = c0; c < c0 + 32; c += 16) {
         float v[16];
         tc_ld16(tW + c, v);
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = gelu_f(v[i] + bias[c + i]);
-        st_bf16x8(sm + kPC + prow(tid, 0, c >> 3), v);
-        st_bf16x8(sm + kPC + prow(tid, 0, (c >> 3) + 1), v + 8);
+        st_bf16x8(sm + kPC + prow(trow, 0, c >> 3), v);
+        st_bf16x8(sm + kPC + prow(trow, 0, (c >> 3) + 1), v + 8);
       }
     }
     handoff();
@@ -284,13 +276,13 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     // ---- H2 = gelu(Z2 + b2) -> PB
     if (!failed) {
 #pragma unroll
-      for (int c = 0; c < 64; c += 16) {
+      for (int c = c0; c < c0 + 32; c += 16) {
         float v[16];
         tc_ld16(tZ2 + c, v);
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = gelu_f(v[i] + bias[64 + c + i]);
-        st_bf16x8(sm + kPB + prow(tid, 0, c >> 3), v);
-        st_bf16x8(sm + kPB + prow(tid, 0, (c >> 3) + 1), v + 8);
+        st_bf16x8(sm + kPB + prow(trow, 0, c >> 3), v);
+        st_bf16x8(sm + kPB + prow(trow, 0, (c >> 3) + 1), v + 8);
       }
     }
     handoff();
@@ -303,16 +295,16 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     commit_wait();
     // ---- Y, residual, dY
     float yv[4] = {0.f, 0.f, 0.f, 0.f};
-    if (!failed) tc_ld4(tW, yv);
+    if (!failed && half == 0) tc_ld4(tW, yv);
 #pragma unroll
     for (int o = 0; o < 4; ++o) yv[o] += bias[128 + o];
     if (!TRAIN) {
-      if (valid && !failed)
+      if (valid && !failed && half == 0)
         *reinterpret_cast<float4*>(a.y + row * 4) = make_float4(yv[0], yv[1], yv[2], yv[3]);
       handoff();  // this tile's TMEM reads done before the next tile's products
       continue;
     }
-    {
+    if (half == 0) {
       const float tt[4] = {tcur.x, tcur.y, tcur.z, tcur.w};
       float dy[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -322,8 +314,8 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
         dy[o] = a.dy_scale * r;
       }
       const float zero8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      st_bf16x8(sm + kPC + prow(tid, kDYoff, 0), dy);
-      st_bf16x8(sm + kPC + prow(tid, kDYoff, 1), zero8);
+      st_bf16x8(sm + kPC + prow(trow, kDYoff, 0), dy);
+      st_bf16x8(sm + kPC + prow(trow, kDYoff, 1), zero8);
     }
     handoff();
     if (tid == 0 && !failed) {
@@ -341,14 +333,14 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     // ---- dZ2 = dH2 . gelu'(Z2 + b2) -> PA (first half)
     if (!failed) {
 #pragma unroll
-      for (int c = 0; c < 64; c += 16) {
+      for (int c = c0; c < c0 + 32; c += 16) {
         float g[16], z[16];
         tc_ld16(tW + c, g);
         tc_ld16(tZ2 + c, z);
 #pragma unroll
         for (int i = 0; i < 16; ++i) g[i] *= gelu_prime_f(z[i] + bias[64 + c + i]);
-        st_bf16x8(sm + kPA + prow(tid, 0, c >> 3), g);
-        st_bf16x8(sm + kPA + prow(tid, 0, (c >> 3) + 1), g + 8);
+        st_bf16x8(sm + kPA + prow(trow, 0, c >> 3), g);
+        st_bf16x8(sm + kPA + prow(trow, 0, (c >> 3) + 1), g + 8);
       }
     }
     handoff();
@@ -364,14 +356,14 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     // ---- dZ1 = dH1 . gelu'(Z1 + b1) -> PA (second half)
     if (!failed) {
 #pragma unroll
-      for (int c = 0; c < 64; c += 16) {
+      for (int c = c0; c < c0 + 32; c += 16) {
         float g[16], z[16];
         tc_ld16(tZ2 + c, g);
         tc_ld16(tW + c, z);
 #pragma unroll
         for (int i = 0; i < 16; ++i) g[i] *= gelu_prime_f(z[i] + bias[c + i]);
-        st_bf16x8(sm + kPA + prow(tid, 1024, c >> 3), g);
-        st_bf16x8(sm + kPA + prow(tid, 1024, (c >> 3) + 1), g + 8);
+        st_bf16x8(sm + kPA + prow(trow, 1024, c >> 3), g);
+        st_bf16x8(sm + kPA + prow(trow, 1024, (c >> 3) + 1), g + 8);
       }
     }
     handoff();
@@ -395,29 +387,31 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
       tc_ld4(tG3, g3);
       float gb[4];
       tc_ld4(tGA + kGaB, gb);
-      if (warp < 2) {  // rows 0..63: dW2, db2, dW3
+      if ((warp & 3) < 2) {  // rows 0..63: dW2 (a half each), db2, dW3
 #pragma unroll
-        for (int c = 0; c < 64; c += 16) {
+        for (int c = c0; c < c0 + 32; c += 16) {
           float v[16];
           tc_ld16(tGA + c, v);
 #pragma unroll
           for (int i = 0; i < 16; i += 4)
-            *reinterpret_cast<float4*>(pg + kOffW2 + tid * 64 + c + i) =
+            *reinterpret_cast<float4*>(pg + kOffW2 + trow * 64 + c + i) =
                 make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         }
-        pg[kOffB2 + tid] = gb[0];
+        if (half == 0) {
+          pg[kOffB2 + trow] = gb[0];
 #pragma unroll
-        for (int o = 0; o < 4; ++o) pg[kOffW3 + o * 64 + tid] = g3[o];
-      } else {  // rows 64..127: dW1, db1; row 64: db3
+          for (int o = 0; o < 4; ++o) pg[kOffW3 + o * 64 + trow] = g3[o];
+        }
+      } else if (half == 0) {  // rows 64..127: dW1, db1; row 64: db3
         float v[16];
         tc_ld16(tGA + 64, v);
-        const int h = tid - 64;
+        const int h = trow - 64;
 #pragma unroll
         for (int i = 0; i < 16; i += 4)
           *reinterpret_cast<float4*>(pg + kOffW1 + h * 16 + i) =
               make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         pg[kOffB1 + h] = gb[0];
-        if (tid == 64) {
+        if (trow == 64) {
 #pragma unroll
           for (int o = 0; o < 4; ++o) pg[kOffB3 + o] = g3[o];
         }
@@ -425,7 +419,7 @@ __global__ void __launch_bounds__(kRows, 2) mlp_kernel(MlpArgs a) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, o);
-    if ((tid & 31) == 0) red[warp] = loss;
+    if (half == 0 && (tid & 31) == 0) red[warp] = loss;
     __syncthreads();
     if (tid == 0) a.part_loss[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
   }
@@ -546,7 +540,7 @@ cudaError_t launch_net(const fv_mlp_trainer* t, bool train, const float* params,
   a.status = t->status;
   const int grid = mlp_grid(t, batch);
   if (grid_out) *grid_out = grid;
-  return fv::launch_kernel(train ? fv::mlp_kernel<true> : fv::mlp_kernel<false>, grid, fv::kRows,
+  return fv::launch_kernel(train ? fv::mlp_kernel<true> : fv::mlp_kernel<false>, grid, fv::kNT,
                       fv::kSmemBytes, t->stream, early, a);
 }
 
