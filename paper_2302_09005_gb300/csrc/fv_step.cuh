@@ -390,10 +390,18 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
 
 // Patch sizes with a compile-time specialisation, per CTA size: the common
 // sizes for 128 threads, small ones for one or two warps, large ones for 256.
-template <int D, int NT>
+// FP32 3D launches with 256 threads (without a plan, or of 8^3) take the sizes
+// of that CTA's class, 6 to 8, 6 and 8 with faces one by one: the runtime-size
+// path is limited by its index arithmetic (updates: 20,011 patches of 2^3..8^3 295
+// -> 256 us, 5,000 of 8^3 158 -> 129; time steps: 8,000 of 8^3 285 -> 249).  With 2 to
+// 5 specialised as well the code no longer fits the instruction caches (3^3..7^3
+// 362 us where 6 to 8 take 317), nor does it in FP64 with 6 and 8 (2^3..8^3 1.44 ->
+// 1.51 ms).
+template <typename T, int D, int NT>
 __host__ __device__ constexpr bool specialised(int p) {
   if (D == 1) return false;
   if (NT <= 64) return D == 3 ? p == 3 : (p == 3 || p == 5 || p == 8);
+  if (NT >= 256 && D == 3 && sizeof(T) == 4) return p >= 6 && p <= 8;
   if (NT >= 256) return D == 3 ? p == 7 : p == 17;
   return D == 3 ? (p == 3 || p == 5 || p == 7) : (p == 3 || p == 5 || p == 8 || p == 17);
 }
@@ -403,7 +411,7 @@ __device__ __forceinline__ void gather_dispatch(const StepParams<T>& a, int pj,
                                                 const Stage<T>& s, const FaceSrc* fs) {
   if constexpr (!GATHER && D != 1) return;
 #define FV_GH(PP)                                                               \
-  if constexpr (specialised<D, NT>(PP)) {                                       \
+  if constexpr (specialised<T, D, NT>(PP)) {                                    \
     if (pj == PP) return gather_halo<T, D, PP, GATHER, CARRY, NT>(a, pj, s, fs); \
   }
   FV_GH(3)
@@ -507,7 +515,7 @@ __device__ __forceinline__ double sum_diffs(const double* G, const int (&j)[D], 
 // would waste.
 template <typename T, int D, int P, int NT>
 __host__ __device__ constexpr bool kPencilFaces() {
-  return sizeof(T) == 4 && P > 0 && D >= 2;
+  return sizeof(T) == 4 && P > 0 && D >= 2 && (NT < 256 || P == 7 || P == 17);
 }
 
 // Whether the face loop of a compile-time patch size runs in warp slots (one
@@ -865,13 +873,14 @@ __device__ __forceinline__ void patch_dispatch(const StepParams<T>& a, int p, in
                                                unsigned long long& lam_next, Pipe& pp,
                                                const NextPatch<T>& nx) {
 #define FV_PC(PP)                                                                           \
-  if constexpr (specialised<D, NT>(PP)) {                                                   \
+  if constexpr (specialised<T, D, NT>(PP)) {                                                \
     if (p == PP)                                                                            \
       return patch_compute<T, D, PP, GATHER, FUSED, CARRY, NT>(a, p, i, off, st, G, hr, red, \
                                                                 run_max, lam_next, pp, nx); \
   }
   FV_PC(3)
   FV_PC(5)
+  FV_PC(6)
   FV_PC(7)
   FV_PC(8)
   FV_PC(17)
