@@ -631,17 +631,30 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     const bool h0 = lo && b == 0, h1 = hi && b == p + 1;
     const int ic = g.icell_kt(k, h0 ? 0 : (h1 ? p - 1 : b - 1), tr);
     // after p: c, E + p; or E + p and, k + 1 components on (a halo cell: the
-    // next), the wave speed of direction k
-    constexpr bool LF = kLamForm<T, D, CARRY, P>();
-    const T* h = hp + (8 * k + (h1 ? 4 : 0)) * ptr + tr;
-    const T* pu = (h0 || h1) ? h : ip + k * nint + ic;
-    const T* pp_ = (h0 || h1) ? h + ptr : ip + D * nint + ic;
+    // next), the wave speed of direction k.  (Two forms of the same addresses:
+    // FP32 17x17 steps 3.49 -> 3.39 ms with the first, FP64 6^3 steps with a carry
+    // 0.90 -> 0.865 with the second.)
     const int sp = (h0 || h1) ? ptr : nint;
-    const int sw = (h0 || h1) ? 2 * ptr : (LF ? 2 + k : 2) * nint;
-    x.u = pu[0];
-    x.pr = pp_[0];
-    x.c = pp_[LF ? sw : sp];
-    x.e = pp_[LF ? sp : sw];
+    if constexpr (sizeof(T) == 4) {
+      const T* pu = h0 ? hp + 8 * k * ptr + tr
+                       : (h1 ? hp + (8 * k + 4) * ptr + tr : ip + k * nint + ic);
+      const T* pp_ = h0 ? hp + (8 * k + 1) * ptr + tr
+                        : (h1 ? hp + (8 * k + 5) * ptr + tr : ip + D * nint + ic);
+      x.u = pu[0];
+      x.pr = pp_[0];
+      x.c = pp_[sp];
+      x.e = pp_[2 * sp];
+    } else {
+      constexpr bool LF = kLamForm<T, D, CARRY, P>();
+      const T* h = hp + (8 * k + (h1 ? 4 : 0)) * ptr + tr;
+      const T* pu = (h0 || h1) ? h : ip + k * nint + ic;
+      const T* pp_ = (h0 || h1) ? h + ptr : ip + D * nint + ic;
+      const int sw = (h0 || h1) ? 2 * ptr : (LF ? 2 + k : 2) * nint;
+      x.u = pu[0];
+      x.pr = pp_[0];
+      x.c = pp_[LF ? sw : sp];
+      x.e = pp_[LF ? sp : sw];
+    }
   };
   // The flux of face j (k) between cells L and R, stored into G.
   auto flux = [&](const int k, const int j, const CellK& L, const CellK& R,
@@ -800,17 +813,27 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
     int jm[D];
 #pragma unroll
     for (int k = 0; k < D; ++k) jm[k] = g.trans(c, k) + ptr * (c[k] - 1) + k * S * nface;
+    T* dst = dst_base + (int64_t)cid * S;
+    if constexpr (sizeof(T) == 8 && D >= 2 && !FUSED && NT < 256) {
+      // one unknown after the other: five copies of the fixed-point sum in
+      // each patch size's code do not fit the instruction caches where a batch
+      // mixes sizes (FP64 updates: 60,000 patches of 2^3..4^3 935 -> 647 us, 20,000
+      // of 3x3..12x12 328 -> 247; with 256 threads, one specialised size, the loop
+      // loses 1 to 3 %)
+#pragma unroll 1
+      for (int v = 0; v < S; ++v)
+        dst[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
+      continue;
+    }
     T qn[S];
 #pragma unroll
     for (int v = 0; v < S; ++v)
       qn[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
-    T* dst = dst_base + (int64_t)cid * S;
 #pragma unroll
     for (int v = 0; v < S; ++v) dst[v] = qn[v];
     if constexpr (FUSED) {
       // the new state's wave speed, for the next step's CFL condition, and
       // its primitives, for the carry
-      T* po = a.prim_out != nullptr ? a.prim_out + i * a.prim_stride + t : nullptr;
       if constexpr (sizeof(T) == 4) {
         const Prim<T, D> w = primitives<T, D>(qn, a.gm1, a.gamma, bad, ar);
 #pragma unroll
@@ -818,7 +841,8 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
           const unsigned long long lb = order_bits(ar.add(abs_t(w.u[k]), w.c));
           lam_next = lb > lam_next ? lb : lam_next;
         }
-        if (po != nullptr) {
+        if (a.prim_out != nullptr) {
+          T* po = a.prim_out + i * a.prim_stride + t;
 #pragma unroll
           for (int m = 0; m < D; ++m) po[m * nint] = w.u[m];
           po[D * nint] = w.p;
@@ -826,6 +850,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
           po[(D + 2) * nint] = w.ep;
         }
       } else {
+        T* po = a.prim_out != nullptr ? a.prim_out + i * a.prim_stride + t : nullptr;
         // FP64: a cell whose wave speed is certain to lie below one already
         // met by the CTA (wave_bounds) needs no primitives for the maximum;
         // where the carry wants them anyway, the bounds would cost more
