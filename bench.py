@@ -86,29 +86,34 @@ ISSUE_PEAK = 4 * NUM_SMS * 2.07e9
 
 
 def fp64_ops_per_patch(d: int, p: int, mode: str = "carry") -> int:
-    """FP64 pipe operations of one patch in the step kernel (the algorithm's
+    """FP64 pipe operations of one patch in the step kernel (the kernel's
     count, the reciprocal and square root counted as the FP64 operations of
-    their Newton refinements: 3 and 5).
-      primitives of a cell: 3 (1/rho) + d (u) + d (j.u) + 2 (p) + 1 (E+p)
-                            + 2 (c^2) + 5 (sqrt) = 13 + 2d;
+    their Newton steps: 2 each; the flux differences of d >= 2 run on the
+    integer pipe).
+      primitives of a cell: 2 (1/rho) + d (u) + d (j.u) + 2 (p) + 1 (E+p)
+                            + 2 (c^2) + 2 (sqrt) = 9 + 2d;
       face flux G:          2 (a) + 2 (u_L + a, u_R - a) + 1 (p_L + p_R)
                             + 2 (rho) + 2d (momenta) + 4 (energy) = 2d + 11;
-      cell update:          s (2d) (sum of G_+ - G_- over d directions, fma);
-      next-step wave speed: primitives + d adds.
+                            3D without the documented carry: a from the cells'
+                            wave speeds (d adds an interior cell, 1 a face-halo
+                            cell), 2d + 9;
+      cell update:          s (fma); d = 1: 2 s.
     mode "update": primitives of the interior and face-halo cells, faces,
-    update; "step": that plus the next-step wave speed; "carry": the time
-    step with the primitive carry (no conversion of the input state)."""
+    update; "step": the same (the next-step wave speed is evaluated only where
+    FP32 bounds allow a new maximum); "carry": the time step with the
+    documented primitive carry (no conversion of the input state, primitives
+    and wave speeds of the new one)."""
     s = d + 2
     interior = p ** d
     halo = 2 * d * p ** (d - 1)
     faces = d * (p + 1) * p ** (d - 1)
-    prim = 13 + 2 * d
-    ops = faces * (2 * d + 11) + interior * s * 2 * d
-    if mode in ("update", "step"):
-        ops += (interior + halo) * prim
-    if mode in ("step", "carry"):
-        ops += interior * (prim + d)
-    return ops
+    prim = 9 + 2 * d
+    ops = interior * s * (1 if d > 1 else 2)
+    if mode == "carry":
+        return ops + faces * (2 * d + 11) + interior * (prim + d)
+    if d == 3:
+        return ops + faces * (2 * d + 9) + interior * (prim + d) + halo * (prim + 1)
+    return ops + faces * (2 * d + 11) + (interior + halo) * prim
 
 
 def alg_bytes_per_patch(d: int, p: int, itemsize: int, carry: bool = False) -> int:

@@ -98,7 +98,7 @@ def source_hash() -> str:
 # includes); host-side API changes leave its counters valid.
 _STEP_CORE = ("fv_step.cuh", "fv_device.cuh", "fv_ptx.cuh")
 KERNEL_SOURCES = {
-    "step": _STEP_CORE + ("fv_update.cu", "fv_update_f32.cu", "fv_update_nt.cu",
+    "step": _STEP_CORE + ("fv_fxsum.cuh", "fv_update.cu", "fv_update_f32.cu", "fv_update_nt.cu",
                           "fv_update_nt_f32.cu"),
     "march3d": _STEP_CORE + ("fv_march3d.cu", "fv_cell3.cuh", "fv_meta.cuh"),
     "rows2d": _STEP_CORE + ("fv_rows2d.cu", "fv_meta.cuh"),
