@@ -160,7 +160,8 @@ inline int64_t patch_faces(int d, int p) {
 // the sizes between its classes refined (us per step, 6 M cells, by threads 32 /
 // 64 / 128 / 256: 3D 4^3 1503 / 1261 / 1518 / 2267; 2D 10x10 782 / 745 / 813 / 1176,
 // 12x12 805 / 715 / 780 / 1030, 14x14 915 / 743 / 733 / 880, 20x20 1564 / 966 / 769 /
-// 729, 24x24 2262 / 1245 / 891 / 749; elsewhere default_nt() was the fastest), and doubled
+// 729, 24x24 2262 / 1245 / 891 / 749; 8x8 703 / 691, but 1,600
+// of them 19.9 / 22.6 us: a warp; elsewhere default_nt() was the fastest), and doubled
 // while the launch still fits once into 384 (FP64) or 128 (FP32) threads per
 // SM and a patch has faces for more lanes.  A small batch is one chain of a
 // patch's phases, and more warps shorten each phase: 64 patches of 8x8, FP64,
@@ -174,7 +175,7 @@ inline int untuned_nt(const fv_batch* h, int p, int64_t count) {
   if (h->d == 1) return nt;
   if (h->prec == FV_FP64) {
     if (h->d == 3 && p == 4) nt = 64;
-    if (h->d == 2 && p >= 8) nt = p <= 12 ? 64 : p < 20 ? 128 : 256;
+    if (h->d == 2 && p >= 9) nt = p <= 12 ? 64 : p < 20 ? 128 : 256;
   }
   const int64_t room = (int64_t)h->num_sms * (h->prec == FV_FP64 ? 384 : 128);
   while (nt < 256 && nt < patch_faces(h->d, p) && 2 * nt * count <= room) nt *= 2;

@@ -10,7 +10,7 @@ from tests import fvtest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,p", [(2, 7), (2, 8), (2, 12), (2, 13), (2, 19), (2, 20), (2, 24),
+@pytest.mark.parametrize("d,p", [(2, 7), (2, 8), (2, 9), (2, 12), (2, 13), (2, 19), (2, 20), (2, 24),
                                  (3, 3), (3, 4), (3, 5), (3, 6), (3, 7), (3, 8)])
 @pytest.mark.parametrize("n", [7, 1300])
 @pytest.mark.parametrize("prec", [0, 1])
