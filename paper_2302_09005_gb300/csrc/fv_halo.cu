@@ -17,9 +17,9 @@ namespace fv {
 template <typename T>
 struct HaloParams {
   T* q;
-  const int64_t* __restrict__ off;
-  const int32_t* __restrict__ sizes;
-  const int32_t* __restrict__ nbr;
+  const int64_t* off;
+  const int32_t* sizes;
+  const int32_t* nbr;
   int64_t n;
   int halo;
   int pmax;
@@ -56,22 +56,6 @@ __device__ __forceinline__ void store_cell(T* dst, const T (&v)[S]) {
   }
 }
 
-// The S unknowns of one cell (16-byte aligned when S sizeof(T) is a multiple
-// of 16, as patch offsets are multiples of 16 bytes), through the read-only
-// path: the cells a halo fill reads are interior cells, which it never writes.
-template <typename T, int S>
-__device__ __forceinline__ void load_cell_ro(const T* src, T (&v)[S]) {
-  if constexpr ((S * sizeof(T)) % 16 == 0) {
-#pragma unroll
-    for (int u = 0; u < (int)(S * sizeof(T) / 16); ++u) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(src) + u);
-      memcpy(&v[u * (16 / sizeof(T))], &w, 16);
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < S; ++u) v[u] = __ldg(src + u);
-  }
-}
 // v[u] = -v[u] for u == neg (selects, so v stays in registers).
 template <typename T, int S>
 __device__ __forceinline__ void negate_comp(T (&v)[S], int neg) {
@@ -220,8 +204,7 @@ __device__ __forceinline__ int64_t halo_src(int t, int p, int h, int per_face, i
 // lanes 0 .. 5 resolve the sources of the patch's faces once (neighbour,
 // outflow, wall) and share them by shuffles, the next patch's size, offset
 // and neighbours are loaded while the current one is copied, and each lane
-// keeps two cells in flight (both loads, through the read-only path, before
-// both stores).  FP64 5^3 patches: 1.76 ms against 2.09 for 262,144 patches;
+// keeps two cells in flight (both loads before both stores).  FP64 5^3 patches: 1.76 ms against 2.09 for 262,144 patches;
 // on 5x5 patches (one pass) it measured slower, so 1D and 2D use halo_kernel.
 template <typename T, int D>
 __global__ void __launch_bounds__(FV_NT) halo_kernel_pipe(HaloParams<T> a) {
@@ -290,8 +273,7 @@ __global__ void __launch_bounds__(FV_NT) halo_kernel_pipe(HaloParams<T> a) {
     const int per_face = h * ptr;
     const int total = NF * per_face;
     T* Q = a.q + off;
-    // two cells per lane in flight: both loads (read-only: the kernel writes
-    // halo cells only and reads interior cells only) before both stores
+    // two cells per lane in flight: both loads before both stores
     for (int t = lane; t < total; t += 64) {
       int64_t d0 = 0, d1 = 0;
       int n0 = -1, n1 = -1;
@@ -299,8 +281,8 @@ __global__ void __launch_bounds__(FV_NT) halo_kernel_pipe(HaloParams<T> a) {
       const int64_t s1 =
           t + 32 < total ? halo_src<D>(t + 32, p, h, per_face, ptr, ne, soff, smode, d1, n1) : -1;
       T v0[S], v1[S];
-      if (s0 >= 0) load_cell_ro<T, S>(a.q + s0, v0);
-      if (s1 >= 0) load_cell_ro<T, S>(a.q + s1, v1);
+      if (s0 >= 0) copy_cell<T, S>(a.q + s0, v0);
+      if (s1 >= 0) copy_cell<T, S>(a.q + s1, v1);
       if (s0 >= 0) {
         negate_comp<T, S>(v0, n0);
         store_cell<T, S>(Q + d0, v0);

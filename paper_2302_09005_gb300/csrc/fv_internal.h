@@ -264,7 +264,10 @@ cudaError_t launch_selftest_math(const double* x, double* out, int64_t n, int wh
 // launch).  Every kernel launched so waits (grid_dep_wait) before it reads or
 // writes anything in global memory but its own unchanging inputs, so the order
 // of the stream holds for everything that is visible; what overlaps is the
-// launch itself.
+// launch itself.  What an earlier kernel may have written (states, metadata,
+// wave speeds) it reads with ordinary loads: the wait orders those, but not the
+// non-coherent path (__ldg, and __restrict__ pointers to const, which let the
+// compiler take it), whose data may not change while the kernel is resident.
 //
 // starts_early: the rule for the patch kernels, at most 256 threads per SM.  A
 // launch that leaves the GPU mostly empty is bound by launch latency (an update

@@ -18,9 +18,9 @@ namespace fv {
 // ---------------------------------------------------------------------------
 template <typename T>
 struct EigParams {
-  const T* __restrict__ q;
-  const int64_t* __restrict__ off;
-  const int32_t* __restrict__ sizes;
+  const T* q;
+  const int64_t* off;
+  const int32_t* sizes;
   int64_t n;
   int halo;
   int pmax;
@@ -74,12 +74,12 @@ __device__ __forceinline__ void eig_load(const T* src, T (&q)[S]) {
   if constexpr ((S * sizeof(T)) % 16 == 0) {
 #pragma unroll
     for (int u = 0; u < (int)(S * sizeof(T) / 16); ++u) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(src) + u);
+      const uint4 w = reinterpret_cast<const uint4*>(src)[u];
       memcpy(&q[u * (16 / sizeof(T))], &w, 16);
     }
   } else {
 #pragma unroll
-    for (int v = 0; v < S; ++v) q[v] = __ldg(src + v);
+    for (int v = 0; v < S; ++v) q[v] = src[v];
   }
 }
 // The largest |u_k| + c of a cell (over every k, or kdir alone), as bits.
@@ -298,9 +298,9 @@ cudaError_t launch_eig_finish(const fv_batch* h, const unsigned long long* parti
 // ---------------------------------------------------------------------------
 template <typename T>
 struct SumParams {
-  const T* __restrict__ q;
-  const int64_t* __restrict__ off;
-  const int32_t* __restrict__ sizes;
+  const T* q;
+  const int64_t* off;
+  const int32_t* sizes;
   int64_t n;
   int halo;
   int pmax;
@@ -414,7 +414,7 @@ __device__ __forceinline__ bool patch_sum(const SumParams<T>& a, int p, int64_t 
         for (int k = D - 2; k >= 0; --k) cid = cid * ne + c[k];
         const T* qc = a.q + off + cid * S;
 #pragma unroll
-        for (int k = 0; k < S; ++k) v[m][k] = __ldg(qc + k);
+        for (int k = 0; k < S; ++k) v[m][k] = qc[k];
       }
     }
     const bool head = t0 < 128;  // the first round starts the sums
@@ -599,8 +599,7 @@ cudaError_t launch_zero_word(unsigned long long* p, cudaStream_t stream) {
 // ---------------------------------------------------------------------------
 // Self-test of the FP64 reciprocal and square root used by the kernels.
 // ---------------------------------------------------------------------------
-__global__ void selftest_math_kernel(const double* __restrict__ x, double* __restrict__ out,
-                                     int64_t n, int which) {
+__global__ void selftest_math_kernel(const double* x, double* out, int64_t n, int which) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     out[i] = which == 0 ? recip(x[i]) : sqrt_t(x[i]);

@@ -58,12 +58,12 @@ namespace fv {
 
 template <typename T>
 struct StepParams {
-  const T* __restrict__ in;
-  T* __restrict__ out;
-  const int64_t* __restrict__ off;
-  const int32_t* __restrict__ sizes;
-  const int32_t* __restrict__ nbr;  // time-step modes
-  const int32_t* __restrict__ order;  // processing order (patch indices), or null
+  const T* in;
+  T* out;
+  const int64_t* off;
+  const int32_t* sizes;
+  const int32_t* nbr;    // time-step modes
+  const int32_t* order;  // processing order (patch indices), or null
   int64_t i_begin, i_end;             // positions of the sequence this launch runs
   int64_t n;                          // patches in the batch
   int64_t n_elems;
@@ -83,8 +83,8 @@ struct StepParams {
   const double* dx_patch;  // update mode: per-patch cell size (or null: dx)
   double* dt_patch;        // with dx_patch: per-patch dt (input, or output under local CFL)
   int local_cfl;           // with dx_patch: dt_i = cfl dx_i / (d lambda_i) per patch
-  const T* __restrict__ prim_in;  // carried primitives of `in` (primitive-carry mode)
-  T* __restrict__ prim_out;       // primitives of `out` (time-step modes), or null
+  const T* prim_in;               // carried primitives of `in` (primitive-carry mode)
+  T* prim_out;                    // primitives of `out` (time-step modes), or null
   int prim_own;                   // 3D FP64: prim_out in fv_run_steps' own form (kCarryOwn)
   int64_t prim_stride;            // elements per patch of prim_in / prim_out
   long long wait_limit = FV_WAIT_LIMIT;  // cycles of a wait for a patch's copy
@@ -346,11 +346,11 @@ __device__ __forceinline__ void gather_halo(const StepParams<T>& a, int pj, cons
 #pragma unroll
       for (int v = 0; v < S; ++v) {
         if (v == 1 + k)
-          dst[v] = neg_t(__ldg(src + v));
+          dst[v] = neg_t(src[v]);
         else
           cp_async_elem(dst + v, src + v);
       }
-      if constexpr (CARRY != kCarryNone) pd[0] = neg_t(__ldg(ps + k * g.nint()));
+      if constexpr (CARRY != kCarryNone) pd[0] = neg_t(ps[k * g.nint()]);
     }
     if constexpr (CARRY != kCarryNone) {
       cp_async_elem(pd + ptr, ps + D * g.nint());
