@@ -271,8 +271,9 @@ __device__ __forceinline__ Prim<T, D> primitives(const T* q, T gm1, T gamma, boo
 // those need the FP64 primitives (19 operations on the scarce pipe; the
 // bounds cost none).  um is |u_k| (kdir = k) or the largest |u_k| (kdir < 0),
 // and lo <= um + c <= hi for the FP64 um + c; false (lo = 0, hi = inf) where
-// that cannot be told: values outside the floats' range, NaN, or a pressure
-// that is not certain to be positive -- the caller evaluates those cells.
+// that cannot be told: values outside the floats' range, NaN, a pressure that
+// is not certain to be positive, or a squared sound speed next to the ends of
+// the floats' range -- the caller evaluates those cells.
 //
 // With x ~ y (1 +- 2^-23) for every truncated input and 2^-23 for the
 // approximate reciprocal, u is within 2^-21 of j / rho, the kinetic energy ke
@@ -315,6 +316,9 @@ __device__ __forceinline__ bool wave_bounds(const double* q, float gm1, float ga
   const float th = E - ke, tot = E + ke, g = gamma * gm1 * inv;
   ok = ok && th > tot * kWaveEps;  // p > 0 for certain (false for NaN)
   const float c2 = g * th, e2 = g * tot * kWaveEps;
+  // c2 and its margin normal numbers (the square root takes subnormal ones for
+  // zero) and finite; um may underflow: it is then far below c
+  ok = ok && c2 > 0x1p-100f && c2 < 0x1p100f;
   float ch, cl;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(ch) : "f"(c2 + e2));
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(cl) : "f"(fmaxf(c2 - e2, 0.f)));
