@@ -518,6 +518,32 @@ __host__ __device__ constexpr bool kPencilFaces() {
   return sizeof(T) == 4 && P > 0 && D >= 2 && (NT < 256 || P == 7 || P == 17);
 }
 
+// Whether the update of a cell sums one unknown after the other (a loop) or all
+// at once (unrolled).  FP64: an unrolled cell is S copies of the fixed-point
+// sum, and with such an update in the code of every compile-time size the kernel
+// no longer fits the instruction caches where a launch mixes sizes.  4 M cells
+// without a plan, time step, unrolled / loop: 2x2..8x8 2.77 / 1.93 ms, 2^3..5^3
+// 2.44 / 1.67, 2x2..17x17 1.11 / 0.93; updates of 60,000 patches of 2^3..4^3 935 /
+// 647 us.  Batches of one size lose nothing in 3D (5^3 872 / 862 us) and up to 4 %
+// in 2D (17x17 509 / 522 us; 10x10, 2,000 patches, 45.6 / 47.3), so time steps with
+// 128 threads keep the runtime size, which is one code for most sizes there,
+// unrolled (16x16 607 us, with the loop 629).  With 256 threads there is one
+// compile-time size, and the loop loses 1 to 3 %.
+template <typename T, int D, int P, bool FUSED, int NT>
+__host__ __device__ constexpr bool kLoopSums() {
+  return sizeof(T) == 8 && D >= 2 && NT < 256 && !(FUSED && D == 2 && P == 0 && NT == 128);
+}
+// A patch's state box: read only, but an FP64 time step passes a cell's new state
+// from the loop of its sums to its primitives through it.
+template <typename T, bool WRITE>
+struct BoxPtr {
+  typedef const T* __restrict__ type;
+};
+template <typename T>
+struct BoxPtr<T, true> {
+  typedef T* type;
+};
+
 // Whether the face loop of a compile-time patch size runs in warp slots (one
 // direction per warp and iteration) rather than over all faces flat: when it
 // keeps at least as many lanes busy (to 2 %).
@@ -547,7 +573,7 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
   const int p = g.p;
   const int nface = g.nface(), nint = g.nint(), ptr = g.ptrans();
   const int tid = threadIdx.x;
-  const T* __restrict__ st = cur.box;
+  typename BoxPtr<T, FUSED && sizeof(T) == 8 && (D >= 2)>::type st = cur.box;
   T* ip = cur.ip;
   T* hp = cur.hp;
   const Arith<T> ar{a.one, a.mone, a.mzero};
@@ -814,23 +840,24 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
 #pragma unroll
     for (int k = 0; k < D; ++k) jm[k] = g.trans(c, k) + ptr * (c[k] - 1) + k * S * nface;
     T* dst = dst_base + (int64_t)cid * S;
-    if constexpr (sizeof(T) == 8 && D >= 2 && !FUSED && NT < 256) {
-      // one unknown after the other: five copies of the fixed-point sum in
-      // each patch size's code do not fit the instruction caches where a batch
-      // mixes sizes (FP64 updates: 60,000 patches of 2^3..4^3 935 -> 647 us, 20,000
-      // of 3x3..12x12 328 -> 247; with 256 threads, one specialised size, the loop
-      // loses 1 to 3 %)
-#pragma unroll 1
-      for (int v = 0; v < S; ++v)
-        dst[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
-      continue;
-    }
     T qn[S];
+    if constexpr (kLoopSums<T, D, P, FUSED, NT>()) {
+#pragma unroll 1
+      for (int v = 0; v < S; ++v) {
+        const T x = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
+        dst[v] = x;
+        if constexpr (FUSED) st[cid * S + v] = x;
+      }
+      if constexpr (!FUSED) continue;
 #pragma unroll
-    for (int v = 0; v < S; ++v)
-      qn[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
+      for (int v = 0; v < S; ++v) qn[v] = st[cid * S + v];
+    } else {
 #pragma unroll
-    for (int v = 0; v < S; ++v) dst[v] = qn[v];
+      for (int v = 0; v < S; ++v)
+        qn[v] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[cid * S + v]);
+#pragma unroll
+      for (int v = 0; v < S; ++v) dst[v] = qn[v];
+    }
     if constexpr (FUSED) {
       // the new state's wave speed, for the next step's CFL condition, and
       // its primitives, for the carry
