@@ -533,6 +533,17 @@ template <typename T, int D, int P, bool FUSED, int NT>
 __host__ __device__ constexpr bool kLoopSums() {
   return sizeof(T) == 8 && D >= 2 && NT < 256 && !(FUSED && D == 2 && P == 0 && NT == 128);
 }
+// Whether small patches share their update out by (cell, unknown): in CTAs of 256
+// threads, sized for a larger patch, a cell's chain of S fixed-point sums leaves
+// most threads idle.  Patches of at most half as many cells as threads; 4 M cells
+// of 2^3 in a handle for 8^3, update 10.0 -> 7.5 ms (for 6^3 4.63 -> 3.60), 4^3
+// 2.40 -> 2.16; mixes of 2^3..8^3 1.54 -> 1.51.  Time steps gain as much there
+// (12.1 -> 10.6 ms) but their code grows by more: 930 patches of 6^3 66 -> 68 us, so
+// they keep the one form.
+template <typename T, int D, int P, bool FUSED, int NT>
+__host__ __device__ constexpr bool kItemSums() {
+  return sizeof(T) == 8 && D == 3 && P == 0 && NT == 256 && !FUSED;
+}
 // A patch's state box: read only, but an FP64 time step passes a cell's new state
 // from the loop of its sums to its primitives through it.
 template <typename T, bool WRITE>
@@ -827,7 +838,8 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
   T* dst_base = a.out + off;
   float run_floor = 0.f;
   if constexpr (FUSED && sizeof(T) == 8) run_floor = wave_floor(*run_max);
-  for (int t = tid; t < nint; t += NT) {
+  // interior cell t: its cell index in the box, its lower face of every direction
+  auto locate = [&](int t, int (&jm)[D]) -> int {
     int c[3] = {0, 0, 0};
     int r = t;
 #pragma unroll
@@ -836,9 +848,26 @@ __device__ __forceinline__ void patch_compute(const StepParams<T>& a, int p_rt, 
       r /= p;
     }
     const int cid = g.cell(c);
-    int jm[D];
 #pragma unroll
     for (int k = 0; k < D; ++k) jm[k] = g.trans(c, k) + ptr * (c[k] - 1) + k * S * nface;
+    return cid;
+  };
+  bool summed = false;
+  if constexpr (kItemSums<T, D, P, FUSED, NT>()) {
+    summed = 2 * nint <= NT;
+    if (summed) {
+#pragma unroll 1
+      for (int e = tid; e < nint * S; e += NT) {
+        const int v = e / nint;
+        int jm[D];
+        const int q = locate(e - v * nint, jm) * S + v;
+        dst_base[q] = fma(mhr, sum_diffs<D>(G + v * nface, jm, ptr, ar), st[q]);
+      }
+    }
+  }
+  for (int t = summed ? nint : tid; t < nint; t += NT) {
+    int jm[D];
+    const int cid = locate(t, jm);
     T* dst = dst_base + (int64_t)cid * S;
     T qn[S];
     if constexpr (kLoopSums<T, D, P, FUSED, NT>()) {
