@@ -161,8 +161,17 @@ inline int64_t patch_faces(int d, int p) {
 // 64 / 128 / 256: 3D 4^3 1503 / 1261 / 1518 / 2267; 2D 10x10 782 / 745 / 813 / 1176,
 // 12x12 805 / 715 / 780 / 1030, 14x14 915 / 743 / 733 / 880, 20x20 1564 / 966 / 769 /
 // 729, 24x24 2262 / 1245 / 891 / 749; 8x8 703 / 691, but 1,600
-// of them 19.9 / 22.6 us: a warp; elsewhere default_nt() was the fastest), and doubled
-// while the launch still fits once into 384 (FP64) or 128 (FP32) threads per
+// of them 19.9 / 22.6 us: a warp; elsewhere default_nt() was the fastest).  Where the
+// patches' sizes are not known (`known` false: no plan), p is the handle's largest
+// size, and 2D handles of 20 to 22 stay at 128 threads: 256 are faster for patches
+// near that size but slower for small ones (6 M cells in a handle of 20, us per
+// update, 128 / 256 threads: 20x20 739 / 687, 2x2..20x20 946 / 1001, 10x10 1031 /
+// 1134, 5x5 2069 / 2895).  From 23 on shared memory leaves two CTAs per SM at either
+// size, and 256 threads are faster for all but the smallest patches (handle of 24:
+// 2x2..24x24 1145 / 972, 10x10 1393 / 1235, 5x5 3034 / 3227).  The other lines lose
+// nothing to default_nt() at smaller sizes (handle of 12: 8x8 791 us at 128 threads,
+// 739 at 64; 5x5 1253, 1048).
+// The CTA is doubled while the launch still fits once into 384 (FP64) or 128 (FP32) threads per
 // SM and a patch has faces for more lanes.  A small batch is one chain of a
 // patch's phases, and more warps shorten each phase: 64 patches of 8x8, FP64,
 // 50 steps in a graph 0.62 -> 0.44 ms (a warp -> eight per patch); updates of
@@ -170,12 +179,12 @@ inline int64_t patch_faces(int d, int p) {
 // at 600 patches (beyond the line) a warp is as fast.  FP32 phases are short,
 // and past 128 threads per SM more warps cost more than they save (300
 // patches of 5^3: 6.4 us at 128 threads, 8.3 at 256).
-inline int untuned_nt(const fv_batch* h, int p, int64_t count) {
+inline int untuned_nt(const fv_batch* h, int p, int64_t count, bool known) {
   int nt = default_nt(h->d, p);
   if (h->d == 1) return nt;
   if (h->prec == FV_FP64) {
     if (h->d == 3 && p == 4) nt = 64;
-    if (h->d == 2 && p >= 9) nt = p <= 12 ? 64 : p < 20 ? 128 : 256;
+    if (h->d == 2 && p >= 9) nt = p <= 12 ? 64 : p < (known ? 20 : 23) ? 128 : 256;
   }
   const int64_t room = (int64_t)h->num_sms * (h->prec == FV_FP64 ? 384 : 128);
   while (nt < 256 && nt < patch_faces(h->d, p) && 2 * nt * count <= room) nt *= 2;

@@ -1,0 +1,86 @@
+"""CTA sizes that launches really take, read from a captured graph of one call:
+where the sizes of a batch are not known (no plan), a handle for larger 2D
+patches does not take a CTA size that its smaller ones lose by."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2302_09005_gb300 import inputs
+from tests import fvtest
+
+pytestmark = pytest.mark.gpu
+
+
+class KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
+                ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def kernel_threads(stream, call):
+    """Threads per CTA of the kernels that call() launches on the stream."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    vp = ctypes.c_void_p
+
+    def ok(r):
+        assert r == 0, r
+    call()  # the library's own first-use work happens outside the capture
+    stream.synchronize()
+    s = vp(stream.cuda_stream)
+    ok(cu.cuStreamBeginCapture_v2(s, 1))
+    call()
+    graph = vp()
+    ok(cu.cuStreamEndCapture(s, ctypes.byref(graph)))
+    n = ctypes.c_size_t(0)
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (vp * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    out = []
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        ok(cu.cuGraphNodeGetType(vp(node), ctypes.byref(kind)))
+        if kind.value == 0:
+            k = KernelNode()
+            ok(cu.cuGraphKernelNodeGetParams_v2(vp(node), ctypes.byref(k)))
+            out.append(int(k.block[0]))
+    ok(cu.cuGraphDestroy(graph))
+    return out
+
+
+def batch(fv, d, p, n, pmax):
+    torch = fvtest.torch_cuda()
+    stream = torch.cuda.Stream()
+    q, off, sz = inputs.random_batch(n, p, d, seed=1)
+    b = fv.Batch(d, max_patch_size=pmax, stream=stream)
+    x, toff, tsz = fvtest.to_dev(q), fvtest.to_dev(off), fvtest.to_dev(sz)
+    y = x.clone()
+    torch.cuda.synchronize()
+    return b, tsz, stream, lambda: b.update(x, y, toff, tsz, 0.01, 0.001)
+
+
+@pytest.fixture(scope="module")
+def fv():
+    fvtest.ensure_built()
+    fvtest.torch_cuda()
+    from paper_2302_09005_gb300 import fv as fvmod
+    return fvmod
+
+
+@pytest.mark.parametrize("pmax,threads", [(12, 64), (19, 128), (20, 128), (22, 128), (23, 256)])
+def test_unknown_sizes(fv, pmax, threads):
+    b, _, stream, call = batch(fv, 2, 5, 3000, pmax)
+    assert kernel_threads(stream, call) == [threads]
+    b.close()
+
+
+@pytest.mark.parametrize("p,threads", [(12, 64), (19, 128), (20, 256), (22, 256)])
+@pytest.mark.parametrize("classes", [True, False])
+def test_known_sizes(fv, p, threads, classes):
+    b, tsz, stream, call = batch(fv, 2, p, 1000, p)
+    fv.fv_batch_plan(b.h, tsz, 1000)
+    if classes:
+        fv.fv_batch_set_schedule(b.h, fv.FV_SCHED_CLASSES)
+    assert kernel_threads(stream, call) == [threads]
+    b.close()
