@@ -548,11 +548,11 @@ __host__ __device__ constexpr bool kItemSums() {
 // from the loop of its sums to its primitives through it.
 template <typename T, bool WRITE>
 struct BoxPtr {
-  typedef const T* __restrict__ type;
+  using type = const T* __restrict__;  // (in shared memory)
 };
 template <typename T>
 struct BoxPtr<T, true> {
-  typedef T* type;
+  using type = T*;
 };
 
 // Whether the face loop of a compile-time patch size runs in warp slots (one
