@@ -386,15 +386,17 @@ fv_status fv_batch_set_schedule(fv_batch* h, fv_schedule schedule);
 /*
  * Patch-to-thread mapping of the FV_SCHED_CLASSES launches: one CTA advances
  * one patch at a time with `threads` threads (32: a warp per patch, 64, 128
- * or 256: a CTA per patch), set per patch size p (1..max_patch_size).  The
- * default (also of launches without a plan) follows the patch size: 32
- * threads for up to 64 interior cells, 256 for 3D patches above 200 cells,
- * else 128; d = 1 supports 128 only (FV_ERR_UNSUPPORTED otherwise).  Where no
- * size was set, an FP64 launch takes 64 threads for 3D patches of 4^3 and 2D
- * ones of 9^2..12^2 and 256 for 2D ones from 20^2 on (without a plan, by
- * max_patch_size: from 23 on), and a launch of so few patches that most of the
- * GPU would stay idle up to 256 threads a patch.  The mapping never changes the
- * results (bitwise).  fv_batch_class_threads reads the current choice.
+ * or 256: a CTA per patch), set per patch size p (1..max_patch_size) here or by
+ * fv_batch_autotune; 0 takes a setting back.  The default (also of launches
+ * without a plan) follows the patch size: 32 threads for up to 64 interior
+ * cells, 256 for 3D patches above 200 cells, else 128; d = 1 supports 128 only
+ * (FV_ERR_UNSUPPORTED otherwise).  Where no size was set, a launch departs from
+ * the default by precision and batch: an FP64 launch takes 64 threads for 3D
+ * patches of 4^3 and 2D ones of 9^2..12^2 and 256 for 2D ones from 20^2 on
+ * (without a plan, by max_patch_size: from 23 on), and a launch of so few
+ * patches that most of the GPU would stay idle up to 256 threads a patch.  The
+ * mapping never changes the results (bitwise).  fv_batch_class_threads reads
+ * the size set, or the default where none is.
  */
 fv_status fv_batch_set_class_threads(fv_batch* h, int p, int threads);
 fv_status fv_batch_class_threads(const fv_batch* h, int p, int* threads);

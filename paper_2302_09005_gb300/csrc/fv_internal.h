@@ -50,7 +50,7 @@ struct fv_batch {
   int64_t cls_begin[64] = {0}, cls_end[64] = {0};
   int occ_cache[4][64][4] = {{{0}}};         // CTAs per SM by (kernel mode, p, CTA size)
   int stage_cache[4][64][4] = {{{0}}};       // and their shared-memory stages
-  int cls_nt[64] = {0};                      // CTA size of the size-class launches (0: 128)
+  int cls_nt[64] = {0};                      // CTA size of the size-class launches (0: untuned_nt)
   int cls_only = -1;                         // autotuner: launch only this class (-1: all)
   int cls_real[64] = {0};                    // class c holds one valid size (not the rejects)
   int occ_one[8][3] = {};                    // CTAs per SM of the FP32 one-size kernels, by p and mode

@@ -237,7 +237,10 @@ fv_status fv_batch_set_class_threads(fv_batch* h, int p, int threads) {
   if (!h) return FV_ERR_INVALID_ARG;
   if (p < 1 || p > h->max_patch_size || p >= 64)
     return sched_err(h, FV_ERR_INVALID_ARG, "patch size outside 1..max_patch_size");
-  if (threads == 0) threads = fv::default_nt(h->d, p);
+  if (threads == 0) {  // back to each launch's own choice
+    h->cls_nt[p] = 0;
+    return FV_OK;
+  }
   if (!fv::valid_nt(threads)) return sched_err(h, FV_ERR_INVALID_ARG, "threads: 32, 64, 128, 256");
   if (h->d == 1 && threads != 128) return sched_err(h, FV_ERR_UNSUPPORTED, "d = 1: 128 threads");
   h->cls_nt[p] = threads;

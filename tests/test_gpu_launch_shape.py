@@ -1,6 +1,7 @@
 """CTA sizes that launches really take, read from a captured graph of one call:
 where the sizes of a batch are not known (no plan), a handle for larger 2D
-patches does not take a CTA size that its smaller ones lose by."""
+patches does not take a CTA size that its smaller ones lose by; a class whose
+CTA size was set goes back to the launch's own choice with 0."""
 import ctypes
 
 import numpy as np
@@ -83,4 +84,18 @@ def test_known_sizes(fv, p, threads, classes):
     if classes:
         fv.fv_batch_set_schedule(b.h, fv.FV_SCHED_CLASSES)
     assert kernel_threads(stream, call) == [threads]
+    b.close()
+
+
+def test_zero_takes_the_launchs_own_choice(fv):
+    b, tsz, stream, call = batch(fv, 3, 4, 3000, 4)
+    fv.fv_batch_plan(b.h, tsz, 3000)
+    fv.fv_batch_set_schedule(b.h, fv.FV_SCHED_CLASSES)
+    own = kernel_threads(stream, call)
+    assert own == [64]
+    default = fv.fv_batch_class_threads(b.h, 4)
+    fv.fv_batch_set_class_threads(b.h, 4, 128)
+    assert kernel_threads(stream, call) == [128] and fv.fv_batch_class_threads(b.h, 4) == 128
+    fv.fv_batch_set_class_threads(b.h, 4, 0)
+    assert kernel_threads(stream, call) == own and fv.fv_batch_class_threads(b.h, 4) == default
     b.close()
