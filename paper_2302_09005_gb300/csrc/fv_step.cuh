@@ -975,7 +975,9 @@ __device__ __forceinline__ void patch_dispatch(const StepParams<T>& a, int p, in
 // at 5 (102 registers): the integer work of the update (fv_fxsum.cuh) runs
 // beside the FP64 work of the other resident CTAs, so more of them fill both
 // pipes (262,144 patches of 5^3 with the carry: 6.34 ms at 5 CTAs, 6.61 at 4,
-// 7.53 at 3; with the sums on the FP64 pipe 7.87 at 5 and 7.98 at 3).
+// 7.53 at 3; with the sums on the FP64 pipe 7.87 at 5 and 7.98 at 3).  The one
+// kernel that does not quite fit is the 3D time step without a carry: it spills 12
+// bytes a thread.
 #ifndef FV_MINBLOCKS_FP64
 #define FV_MINBLOCKS_FP64 5
 #endif
