@@ -26,6 +26,7 @@
 #include <new>
 #include <vector>
 
+#include "fv_chunks.h"
 #include "fv_internal.h"
 
 constexpr int kHostSlots = 3;
@@ -168,32 +169,25 @@ fv_status fv_patch_update_host(fv_batch* h, const void* host_in, void* host_out,
       return herr(h, FV_ERR_INVALID_ARG, "patch offsets must ascend without overlap");
   }
   const bool inplace = host_in == host_out;
-  int64_t chunk = chunk_patches;
-  if (chunk <= 0) {
-    // an eighth of the batch, 4 to 256 MB: the copy in, the update and the
-    // copy out overlap only from chunk to chunk, and a chunk costs the host
-    // some 20 us.  One chunk / eighths, us per call: 94.6 MB (8,192 2D
-    // patches of 17x17, FP64) 1299 / 876, 31.4 MB 660 / 596, 450 MB 4591 /
-    // 2847; 5.9 MB 121 / 99 in two, 155 in eight; 3.6 GB in 256 MB chunks
-    // 19.8 ms, in 128 MB chunks 20.3.
-    const int64_t per = len(0) * (int64_t)es;
-    int64_t want = (off[n - 1] + len(n - 1) - off[0]) * (int64_t)es / 8;
-    if (want < (4ll << 20)) want = 4ll << 20;
-    if (want > (256ll << 20)) want = 256ll << 20;
-    chunk = want / (per > 0 ? per : 1);
-    if (chunk < 1) chunk = 1;
-  }
-  if (chunk > n) chunk = n;
-  const int64_t nchunks = (n + chunk - 1) / chunk;
-  // the largest chunk in bytes (16-byte rounded)
+  // chunks of chunk_patches patches, or by bytes
+  const int64_t want =
+      chunk_patches > 0 ? 0 : fv::chunk_bytes((off[n - 1] + len(n - 1) - off[0]) * (int64_t)es);
+  auto end_of = [&](int64_t p0) -> int64_t {
+    if (chunk_patches > 0) return n - p0 < chunk_patches ? n : p0 + chunk_patches;
+    return fv::chunk_end(p0, n, off, len, (int64_t)es, want);
+  };
+  // the largest chunk in patches and in bytes (16-byte rounded)
+  int64_t maxn = 0;
   size_t maxb = 0;
-  for (int64_t c = 0; c < nchunks; ++c) {
-    const int64_t p0 = c * chunk, p1 = p0 + chunk < n ? p0 + chunk : n;
+  for (int64_t p0 = 0; p0 < n;) {
+    const int64_t p1 = end_of(p0);
     const size_t b = (size_t)(off[p1 - 1] + len(p1 - 1) - off[p0]) * es;
     maxb = b > maxb ? b : maxb;
+    maxn = p1 - p0 > maxn ? p1 - p0 : maxn;
+    p0 = p1;
   }
   maxb = (maxb + 15) & ~(size_t)15;
-  cudaError_t e = stage_reserve(h, maxb, chunk);
+  cudaError_t e = stage_reserve(h, maxb, maxn);
   if (e != cudaSuccess) return herr(h, FV_ERR_CUDA, cudaGetErrorString(e));
   auto* st = static_cast<fv_host_stage*>(h->host_stage);
   // the spans of a patch, [lo, hi) in elements of its box: in (what the
@@ -207,9 +201,9 @@ fv_status fv_patch_update_host(fv_batch* h, const void* host_in, void* host_out,
   // the chunks start once the work already on the handle's stream is done
   e = cudaEventRecord(st->ev_comp[0], h->stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st->h2d, st->ev_comp[0], 0);
-  for (int64_t c = 0; c < nchunks && e == cudaSuccess; ++c) {
+  for (int64_t c = 0, p0 = 0, p1 = 0; p0 < n && e == cudaSuccess; ++c, p0 = p1) {
     const int k = (int)(c % kHostSlots);
-    const int64_t p0 = c * chunk, p1 = p0 + chunk < n ? p0 + chunk : n;
+    p1 = end_of(p0);
     const int64_t nc = p1 - p0;
     const int64_t base = off[p0];
     const size_t bytes = (size_t)(off[p1 - 1] + len(p1 - 1) - base) * es;
