@@ -177,8 +177,9 @@ fv_status fv_max_eigenvalue_reduce(fv_batch* h, const void* q_with_halo,
  * fv_patch_update_host -- fv_patch_update_batch on patches in HOST memory:
  * the paper's offload pattern (the engine ships a batch of patches with
  * their halos to the GPU for every update and takes the results back).  The
- * batch is cut into chunks of chunk_patches consecutive patches (<= 0: an
- * eighth of the batch, 4 to 256 MB); the copy in of a chunk, the update of
+ * batch is cut into chunks of chunk_patches consecutive patches (<= 0: by
+ * bytes, an eighth of the batch, 4 to 256 MB; 256 MB where the host memory is
+ * not pinned, whose copies do not overlap); the copy in of a chunk, the update of
  * the previous one and the copy out of the one before overlap (two copy
  * streams, the handle's stream for the update, three device staging slots the
  * handle keeps until fv_batch_destroy).

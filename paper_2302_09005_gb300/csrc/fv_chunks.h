@@ -9,14 +9,17 @@
 
 namespace fv {
 
-// Bytes of a chunk: an eighth of the batch, 4 to 256 MB.  The copy in, the
-// update and the copy out overlap only from chunk to chunk, and a chunk costs
-// the host some 20 us.  One chunk / eighths, us per call: 94.6 MB (8,192 2D
+// Bytes of a chunk: on pinned memory an eighth of the batch, 4 to 256 MB.  The
+// copy in, the update and the copy out overlap only from chunk to chunk, and a
+// chunk costs the host some 20 us.  One chunk / eighths, us per call: 94.6 MB (8,192 2D
 // patches of 17x17, FP64) 1299 / 876, 31.4 MB 660 / 596, 450 MB 4591 / 2847;
 // 5.9 MB 121 / 99 in two, 155 in eight; 3.6 GB in 256 MB chunks 19.8 ms, in
-// 128 MB chunks 20.3.
-inline int64_t chunk_bytes(int64_t batch_bytes) {
-  const int64_t lo = 4ll << 20, hi = 256ll << 20, want = batch_bytes / 8;
+// 128 MB chunks 20.3.  Copies of pageable memory hold the calling thread and do
+// not overlap, so there only the cost of a chunk is left: 256 MB always (256 MB /
+// eighths, us per call in place: 5.9 MB 123 / 164, 56 MB 608 / 1131, 94.6 MB 1237 /
+// 1566, 450 MB 4331 / 4826).
+inline int64_t chunk_bytes(int64_t batch_bytes, bool pinned) {
+  const int64_t lo = 4ll << 20, hi = 256ll << 20, want = pinned ? batch_bytes / 8 : hi;
   return want < lo ? lo : want > hi ? hi : want;
 }
 

@@ -79,6 +79,17 @@ fv_status herr(fv_batch* h, fv_status st, const char* msg) {
   return st;
 }
 
+// Whether copies from and to p run beside the calling thread: not for pageable
+// host memory, which the driver does not know.
+bool copies_async(const void* p) {
+  cudaPointerAttributes at = {};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type != cudaMemoryTypeUnregistered;
+}
+
 // Grows the staging of a handle to chunks of `bytes` bytes and `npatch`
 // patches (never shrinks).
 cudaError_t stage_reserve(fv_batch* h, size_t bytes, int64_t npatch) {
@@ -170,8 +181,10 @@ fv_status fv_patch_update_host(fv_batch* h, const void* host_in, void* host_out,
   }
   const bool inplace = host_in == host_out;
   // chunks of chunk_patches patches, or by bytes
-  const int64_t want =
-      chunk_patches > 0 ? 0 : fv::chunk_bytes((off[n - 1] + len(n - 1) - off[0]) * (int64_t)es);
+  int64_t want = 0;
+  if (chunk_patches <= 0)
+    want = fv::chunk_bytes((off[n - 1] + len(n - 1) - off[0]) * (int64_t)es,
+                           copies_async(host_in) && copies_async(host_out));
   auto end_of = [&](int64_t p0) -> int64_t {
     if (chunk_patches > 0) return n - p0 < chunk_patches ? n : p0 + chunk_patches;
     return fv::chunk_end(p0, n, off, len, (int64_t)es, want);

@@ -12,7 +12,7 @@ from paper_2302_09005_gb300 import _build
 
 SRC = """
 #include "fv_chunks.h"
-extern "C" int64_t bytes_of(int64_t b) { return fv::chunk_bytes(b); }
+extern "C" int64_t bytes_of(int64_t b, int pinned) { return fv::chunk_bytes(b, pinned != 0); }
 extern "C" int64_t end_of(int64_t p0, int64_t n, const int64_t* off, const int64_t* len, int64_t es,
                           int64_t want) {
   return fv::chunk_end(p0, n, off, [&](int64_t i) { return len[i]; }, es, want);
@@ -29,7 +29,7 @@ def lib(tmp_path_factory):
                     str(d / "t.cpp"), "-o", so], check=True)
     lb = ctypes.CDLL(so)
     lb.bytes_of.restype = lb.end_of.restype = ctypes.c_int64
-    lb.bytes_of.argtypes = [ctypes.c_int64]
+    lb.bytes_of.argtypes = [ctypes.c_int64, ctypes.c_int]
     lb.end_of.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p,
                           ctypes.c_int64, ctypes.c_int64]
     return lb
@@ -68,5 +68,6 @@ def test_chunks_by_bytes(lib, kind, gap, want):
 
 def test_chunk_bytes_bounds(lib):
     mb = 1 << 20
-    assert [lib.bytes_of(b) for b in (0, mb, 32 * mb, 80 * mb, 2048 * mb, 1 << 40)] == \
+    assert [lib.bytes_of(b, 1) for b in (0, mb, 32 * mb, 80 * mb, 2048 * mb, 1 << 40)] == \
         [4 * mb, 4 * mb, 4 * mb, 10 * mb, 256 * mb, 256 * mb]
+    assert [lib.bytes_of(b, 0) for b in (0, 80 * mb, 1 << 40)] == [256 * mb] * 3

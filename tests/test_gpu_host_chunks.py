@@ -51,3 +51,9 @@ def test_staging_follows_the_bytes(fv, first):
     sizes[0] = first
     total, used = run_host(fv, sizes, True)
     assert used <= 3 * (total / 8 + 40000 + 12 * len(sizes)) + 9 * (4 << 20)
+
+
+def test_pageable_memory_goes_in_large_chunks(fv):
+    """Three slots of the whole batch: its copies do not overlap anyway."""
+    total, used = run_host(fv, np.full(1500, 8, dtype=np.int32), False)
+    assert used >= 3 * total
