@@ -174,7 +174,7 @@ fv_status fv_batch_destroy(fv_batch* h) {
   graph_cache_clear(h);
   fv::plan_free(h);
   fv::host_stage_free(h);
-  for (void* pbuf : h->d_prim)
+  for (void* pbuf : h->carry.p)
     if (pbuf) cudaFree(pbuf);
   cudaError_t e2 = cudaFree(h->ws);
   delete h;
@@ -478,32 +478,22 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
     const size_t es = h->prec == FV_FP64 ? 8 : 4;
     const int64_t doc = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size);
     const int64_t full = n * fv::prim_stride_elems(h->d, h->prec, h->max_patch_size, true);
-    // the library's own form, or, where memory does not allow it (3D: a third
-    // more), the documented one
-    if (full > h->prim_cap && !(h->prim_doc && doc <= h->prim_cap)) {
+    if (fv::carry_must_grow(h->carry, full, doc)) {
       cudaError_t e = cudaStreamSynchronize(h->stream);
-      graph_cache_clear(h);
-      h->prim_cap = 0;
-      for (const int64_t need : {full, doc}) {
-        for (void*& pbuf : h->d_prim) {
-          if (pbuf) cudaFree(pbuf);
-          pbuf = nullptr;
-        }
-        if (e == cudaErrorMemoryAllocation) {
-          cudaGetLastError();
-          e = cudaSuccess;
-        }
-        for (void*& pbuf : h->d_prim)
-          if (e == cudaSuccess) e = cudaMalloc(&pbuf, es * (size_t)need);
-        if (e == cudaSuccess) {
-          h->prim_cap = need;
-          h->prim_doc = need < full;
-        }
-        if (e != cudaErrorMemoryAllocation) break;
-      }
       if (e != cudaSuccess) return cuda_err(h, e, "primitive buffers");
+      graph_cache_clear(h);
+      auto alloc = [&](void** p, int64_t elems) {
+        e = cudaMalloc(p, es * (size_t)elems);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+        return e == cudaSuccess                 ? fv::CarryAlloc::Ok
+               : e == cudaErrorMemoryAllocation ? fv::CarryAlloc::NoMemory
+                                                : fv::CarryAlloc::Error;
+      };
+      if (fv::carry_grow(h->carry, full, doc, alloc, [](void* p) { cudaFree(p); }) !=
+          fv::CarryAlloc::Ok)
+        return cuda_err(h, e, "primitive buffers");
     }
-    own = full <= h->prim_cap;
+    own = full <= h->carry.cap;
   }
   auto enqueue = [&]() -> fv_status {
     fv_status s = fv_halo_fill(h, q0, off, sizes, nbr, n);
@@ -513,8 +503,8 @@ fv_status fv_run_steps(fv_batch* h, void* q0, void* q1, const int64_t* off, cons
     void* b = q1;
     for (int k = 0; k < n_steps && s == FV_OK; ++k) {
       // step k reads the primitives step k-1 left and hands on its own
-      const void* pin = (!carry || k == 0) ? nullptr : h->d_prim[(k - 1) & 1];
-      void* pout = (carry && k + 1 < n_steps) ? h->d_prim[k & 1] : nullptr;
+      const void* pin = (!carry || k == 0) ? nullptr : h->carry.p[(k - 1) & 1];
+      void* pout = (carry && k + 1 < n_steps) ? h->carry.p[k & 1] : nullptr;
       s = time_step_impl(h, a, b, off, sizes, nbr, n, dx, cfl, nullptr, nullptr, pin, pout,
                          own);
       std::swap(a, b);

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "fv.h"
+#include "fv_carry.h"
 
 // Threads per CTA of the patch kernels.
 #define FV_NT 128
@@ -35,10 +36,7 @@ struct fv_batch {
   double* d_sum_partials = nullptr;          // FV_MAX_RED_BLOCKS * 8 slots
   unsigned long long* d_queue = nullptr;     // FV_SCHED_QUEUE: positions handed out
   int blocks_per_sm[4][4] = {{0}};           // occupancy by kernel mode and CTA size
-  // primitive carry of fv_run_steps: two buffers of prim_cap elements
-  void* d_prim[2] = {nullptr, nullptr};
-  int64_t prim_cap = 0;
-  bool prim_doc = false;  // in the documented form: the library's own did not fit
+  fv::CarryBuffers carry;                    // primitive carry of fv_run_steps
   void* graph_cache = nullptr;               // captured multi-step graphs
   // schedule (fv_sched.cu): processing order sorted by size, size classes
   int sched = 0;                             // fv_schedule
