@@ -427,6 +427,7 @@ def run_ours(args, ws, rank, local):
                 "unit": "T FP64-pipe ops/s", "frac": achieved / peak_ops,
                 "traffic": _traffic(args.workload),
                 "ops_per_launch": ops,
+                "counts": "FP64 operations only; the flux sums run on the integer pipe",
                 "peak_source": "derived: 2 FP64 lanes/SM x 152 SMs x max SM clock "
                                f"{peaks.get('sm_max_mhz', 2070.0):.0f} MHz"}
     else:

@@ -101,11 +101,14 @@ __device__ __forceinline__ unsigned long long eig_value(const T* q, T gm1, T gam
 // FP64: FP32 bounds of every cell first (wave_bounds), then the FP64 wave
 // speed of the cells whose upper bound reaches the patch's largest lower bound
 // (or, where only the batch maximum is asked for, the warp's largest wave
-// speed so far): usually one cell or two of a patch, so the kernel leaves the
-// FP64 pipe, which bound it when every cell was converted in FP64 (262,144
-// patches of 5^3: 3.08 ms, now 0.82 with the per-patch values and 0.72 without;
-// 40,000 of 7^3: 1.07 -> 0.25).
-// The maximum is exact all the same.
+// speed so far).  Where the states vary from cell to cell that is one cell or
+// two of a patch, and the kernel leaves the FP64 pipe, which bound it when every
+// cell was converted in FP64 (random states, 262,144 patches of 5^3: 3.08 ms,
+// now 0.82 with the per-patch values and 0.72 without; 40,000 of 7^3: 1.07 ->
+// 0.25).  Where the wave speed is constant over a patch every cell is a
+// candidate and is loaded again for FP64: 32,768 patches of 5^3 395 -> 235 us for
+// a uniform moving state, 395 -> 333 for a blast into gas at rest, 108 for random
+// states.  The maximum is exact all the same.
 template <typename T, int D>
 __global__ void __launch_bounds__(FV_NT) eig_kernel(EigParams<T> a) {
   constexpr int S = D + 2;
