@@ -129,8 +129,14 @@ fv_status fv_batch_create(fv_batch** out, int d, int s, const fv_options* o, voi
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   h->smem_optin = smem_optin;
-  if (e == cudaSuccess &&
-      fv::update_smem_bytes(d, h->prec, h->max_patch_size, 1) > (size_t)smem_optin) {
+  // the modes' forms differ in size (with one stage not by CTA size): every mode
+  // takes the largest patches
+  size_t smem = 0;
+  for (int mode : {fv::kModeUpdate, fv::kModePrim}) {
+    const size_t b = fv::update_smem_bytes(d, h->prec, mode, 128, h->max_patch_size, 1);
+    smem = b > smem ? b : smem;
+  }
+  if (e == cudaSuccess && smem > (size_t)smem_optin) {
     delete h;
     return FV_ERR_UNSUPPORTED;  // max_patch_size too large for shared memory
   }

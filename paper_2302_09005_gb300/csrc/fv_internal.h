@@ -125,7 +125,7 @@ inline int64_t prim_stride_elems(int d, fv_precision prec, int pmax, bool own = 
 std::mutex& smem_attr_mutex();
 
 // Shared memory bytes of the update kernel for patches up to pmax.
-size_t update_smem_bytes(int d, fv_precision prec, int pmax, int nstage);
+size_t update_smem_bytes(int d, fv_precision prec, int mode, int nt, int pmax, int nstage);
 cudaError_t launch_update(const fv_batch* h, const UpdateLaunch& a, int grid);
 cudaError_t step_occupancy(const fv_batch* h, int mode, int pmax, int nstage, int nt,
                            int* blocks_per_sm);

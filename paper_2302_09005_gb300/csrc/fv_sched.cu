@@ -43,7 +43,7 @@ void plan_free(fv_batch* h) {
 cudaError_t step_shape(const fv_batch* h, int mode, int pmax, int nt, int* nstage, int* bps) {
   int one = 0, two = 0;
   cudaError_t e = cudaSuccess;
-  if (update_smem_bytes(h->d, h->prec, pmax, 2) <= (size_t)h->smem_optin)
+  if (update_smem_bytes(h->d, h->prec, mode, nt, pmax, 2) <= (size_t)h->smem_optin)
     e = step_occupancy(h, mode, pmax, 2, nt, &two);
   if (e == cudaSuccess) e = step_occupancy(h, mode, pmax, 1, nt, &one);
   *nstage = one > two ? 1 : 2;

@@ -181,7 +181,17 @@ static_assert(kFaceSrcOff + 2 * 6 * (int)sizeof(FaceSrc) <= kHdrBytes, "header t
 // the current one (one stage when two do not fit: the copy of the next
 // patch then starts after the current patch is done).  The face fluxes G
 // follow the stages.
-template <typename T, int D, int CARRY>
+// Primitives that are computed, not copied, are the current patch's alone: in
+// FP64 3D CTAs of 256 threads they follow the stages once, and two stages of 8^3
+// fit (4 M cells, step: 8^3 1093 -> 1011 us, 4^3 in a handle for 8^3 2816 -> 2442,
+// update 2179 -> 1914).  Elsewhere two stages fit as it is; smaller CTAs would
+// only pay for the addresses (2^3, a warp, 1378 -> 1392 us), and in 2D take two
+// stages where one makes as many CTAs resident (2x2 .. 6x6 2.10 -> 2.24 ms).
+template <typename T, int D, int CARRY, int NT>
+constexpr bool kPrimsOnce() {
+  return sizeof(T) == 8 && D == 3 && CARRY == kCarryNone && NT == 256;
+}
+template <typename T, int D, int CARRY, int NT>
 struct Carve {
   int nstage, box, ip, hp, stage, g;
   __host__ __device__ Carve(int pmax, int nstage_)
@@ -189,9 +199,11 @@ struct Carve {
         box(round_up(stage_elems<D>(pmax), 16 / sizeof(T))),
         ip(round_up(iprim_elems<T, D, CARRY>(pmax), 16 / sizeof(T))),
         hp(round_up(hprim_elems<T, D>(pmax), 16 / sizeof(T))),
-        stage(box + ip + hp),
+        stage(kPrimsOnce<T, D, CARRY, NT>() ? box : box + ip + hp),
         g(round_up(gface_elems<D>(pmax), 16 / sizeof(T))) {}
-  __host__ __device__ int total() const { return nstage * stage + g; }
+  __host__ __device__ int total() const {
+    return nstage * stage + (kPrimsOnce<T, D, CARRY, NT>() ? ip + hp : 0) + g;
+  }
 };
 
 template <typename T>
@@ -1001,16 +1013,23 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
   unsigned long long* red = reinterpret_cast<unsigned long long*>(smem_raw + kRedOff);
   unsigned long long* run_max = reinterpret_cast<unsigned long long*>(smem_raw + kRunMaxOff);
   FaceSrc* fsrc = reinterpret_cast<FaceSrc*>(smem_raw + kFaceSrcOff);  // [stage][face]
-  const Carve<T, D, CARRY> cv(a.pmax, a.nstage);
+  const Carve<T, D, CARRY, NT> cv(a.pmax, a.nstage);
   const bool single = a.nstage == 1;
   T* const sbase = reinterpret_cast<T*>(smem_raw + kHdrBytes);
   // stage s (0 or 1; the same one when single), built by arithmetic so the
   // pointers stay in registers
+  constexpr bool once = kPrimsOnce<T, D, CARRY, NT>();
   auto stage_at = [&](int s) -> Stage<T> {
     T* b = sbase + (single ? 0 : s) * cv.stage;
-    return Stage<T>{b, b + cv.box, b + cv.box + cv.ip};
+    if constexpr (once) {
+      T* ip = single ? b + cv.box : sbase + 2 * cv.stage;
+      return Stage<T>{b, ip, ip + cv.ip};
+    } else {
+      return Stage<T>{b, b + cv.box, b + cv.box + cv.ip};
+    }
   };
   T* G = sbase + cv.nstage * cv.stage;
+  if constexpr (once) G += cv.ip + cv.hp;
   const int tid = threadIdx.x;
 
   double dtv;
@@ -1133,9 +1152,9 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
 }
 
 // Bytes of dynamic shared memory of the kernel for patches up to pmax.
-template <typename T, int D, int CARRY>
+template <typename T, int D, int CARRY, int NT>
 inline size_t step_smem_bytes(int pmax, int nstage) {
-  return kHdrBytes + sizeof(T) * (size_t)Carve<T, D, CARRY>(pmax, nstage).total();
+  return kHdrBytes + sizeof(T) * (size_t)Carve<T, D, CARRY, NT>(pmax, nstage).total();
 }
 
 // Raises the kernel's dynamic shared-memory limit on the current device once
@@ -1194,7 +1213,7 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
   a.prim_own = l.prim_own ? 1 : 0;
   a.wait_limit = h->wait_limit;
   a.queue = l.queue;
-  const size_t smem = step_smem_bytes<T, D, CARRY>(l.pmax, a.nstage);
+  const size_t smem = step_smem_bytes<T, D, CARRY, NT>(l.pmax, a.nstage);
   cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
   return launch_kernel(step_kernel<T, D, GATHER, FUSED, CARRY, NT>, grid, NT, smem, h->stream,
@@ -1203,7 +1222,7 @@ static cudaError_t launch_step_t(const fv_batch* h, const UpdateLaunch& l, int g
 
 template <typename T, int D, bool GATHER, bool FUSED, int CARRY, int NT>
 static cudaError_t occupancy_t(int pmax, int nstage, int* bps) {
-  const size_t smem = step_smem_bytes<T, D, CARRY>(pmax, nstage);
+  const size_t smem = step_smem_bytes<T, D, CARRY, NT>(pmax, nstage);
   cudaError_t e = ensure_smem<T, D, GATHER, FUSED, CARRY, NT>(smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(

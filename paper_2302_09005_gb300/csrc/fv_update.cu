@@ -22,21 +22,24 @@ FV_EXTERN(float, 64)
 FV_EXTERN(float, 256)
 #undef FV_EXTERN
 
-template <int D>
-static size_t smem_by_prec(fv_precision prec, int pmax, int nstage) {
-  // the larger of the FP64 modes' forms
-  if (prec == FV_FP64) {
-    const size_t a = step_smem_bytes<double, D, kCarryNone>(pmax, nstage);
-    const size_t b = step_smem_bytes<double, D, kCarryDoc>(pmax, nstage);
-    return a > b ? a : b;
-  }
-  return step_smem_bytes<float, D, kCarryNone>(pmax, nstage);
+template <typename T, int D, int NT>
+static size_t smem_by_mode(int mode, int pmax, int nstage) {
+  if (mode == kModePrim) return step_smem_bytes<T, D, kCarryDoc, NT>(pmax, nstage);
+  if (mode == kModeOwn) return step_smem_bytes<T, D, kCarryOwn, NT>(pmax, nstage);
+  return step_smem_bytes<T, D, kCarryNone, NT>(pmax, nstage);
+}
+template <typename T, int NT>
+static size_t smem_by_d(int d, int mode, int pmax, int nstage) {
+  return d == 1   ? smem_by_mode<T, 1, NT>(mode, pmax, nstage)
+         : d == 2 ? smem_by_mode<T, 2, NT>(mode, pmax, nstage)
+                  : smem_by_mode<T, 3, NT>(mode, pmax, nstage);
 }
 
-size_t update_smem_bytes(int d, fv_precision prec, int pmax, int nstage) {
-  return d == 1   ? smem_by_prec<1>(prec, pmax, nstage)
-         : d == 2 ? smem_by_prec<2>(prec, pmax, nstage)
-                  : smem_by_prec<3>(prec, pmax, nstage);
+// (two layouts: CTAs of 256 threads and smaller ones)
+size_t update_smem_bytes(int d, fv_precision prec, int mode, int nt, int pmax, int nstage) {
+  if (prec == FV_FP32) return smem_by_d<float, 128>(d, mode, pmax, nstage);
+  return nt == 256 ? smem_by_d<double, 256>(d, mode, pmax, nstage)
+                   : smem_by_d<double, 128>(d, mode, pmax, nstage);
 }
 
 template <typename T>
