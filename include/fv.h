@@ -394,10 +394,10 @@ fv_status fv_batch_set_schedule(fv_batch* h, fv_schedule schedule);
  * (FV_ERR_UNSUPPORTED otherwise).  Where no size was set, a launch departs from
  * the default by precision and batch: an FP64 launch takes 64 threads for 3D
  * patches of 4^3 and 2D ones of 9^2..12^2 and 256 for 2D ones from 20^2 on
- * (without a plan, by max_patch_size: from 23 on), and a launch of so few
- * patches that most of the GPU would stay idle up to 256 threads a patch.  The
- * mapping never changes the results (bitwise).  fv_batch_class_threads reads
- * the size set, or the default where none is.
+ * (without a plan, by max_patch_size), and a launch of so few patches that most
+ * of the GPU would stay idle up to 256 threads a patch.  The mapping never
+ * changes the results (bitwise).  fv_batch_class_threads reads the size set, or
+ * the default where none is.
  */
 fv_status fv_batch_set_class_threads(fv_batch* h, int p, int threads);
 fv_status fv_batch_class_threads(const fv_batch* h, int p, int* threads);

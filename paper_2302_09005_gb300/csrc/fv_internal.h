@@ -159,30 +159,27 @@ inline int64_t patch_faces(int d, int p) {
 // 64 / 128 / 256: 3D 4^3 1503 / 1261 / 1518 / 2267; 2D 10x10 782 / 745 / 813 / 1176,
 // 12x12 805 / 715 / 780 / 1030, 14x14 915 / 743 / 733 / 880, 20x20 1564 / 966 / 769 /
 // 729, 24x24 2262 / 1245 / 891 / 749; 8x8 703 / 691, but 1,600
-// of them 19.9 / 22.6 us: a warp; elsewhere default_nt() was the fastest).  Where the
-// patches' sizes are not known (`known` false: no plan), p is the handle's largest
-// size, and 2D handles of 20 to 22 stay at 128 threads: 256 are faster for patches
-// near that size but slower for small ones (6 M cells in a handle of 20, us per
-// update, 128 / 256 threads: 20x20 739 / 687, 2x2..20x20 946 / 1001, 10x10 1031 /
-// 1134, 5x5 2069 / 2895).  From 23 on shared memory leaves two CTAs per SM at either
-// size, and 256 threads are faster for all but the smallest patches (handle of 24:
-// 2x2..24x24 1145 / 972, 10x10 1393 / 1235, 5x5 3034 / 3227).  The other lines lose
-// nothing to default_nt() at smaller sizes (handle of 12: 8x8 791 us at 128 threads,
-// 739 at 64; 5x5 1253, 1048).
-// The CTA is doubled while the launch still fits once into 384 (FP64) or 128 (FP32) threads per
-// SM and a patch has faces for more lanes.  A small batch is one chain of a
+// of them 19.9 / 22.6 us: a warp; elsewhere default_nt() was the fastest).  Without a
+// plan p is the handle's largest size, whatever the batch holds (6 M cells, us per
+// update, default / refined): in a handle of 12 smaller patches gain as well (8x8
+// 791 / 739, 5x5 1253 / 1048), in one of 24 too (2x2..24x24 1145 / 970, 5x5 3034 /
+// 2818, 24x24 864 / 679); in one of 20 small ones pay for the large (20x20 739 / 685,
+// 10x10 1031 / 1045, 2x2..20x20 946 / 987, 5x5 2069 / 2542, which is what they took
+// before the fixed-point sums, 2492).  The CTA is doubled while the launch still
+// fits once into 384 (FP64) or 128 (FP32) threads per SM and a patch has faces
+// for more lanes.  A small batch is one chain of a
 // patch's phases, and more warps shorten each phase: 64 patches of 8x8, FP64,
 // 50 steps in a graph 0.62 -> 0.44 ms (a warp -> eight per patch); updates of
 // 64 patches, FP64, 3^3 12.4 -> 8.2 us, 8x8 12.3 -> 8.2, 17x17 14.4 -> 12.4;
 // at 600 patches (beyond the line) a warp is as fast.  FP32 phases are short,
 // and past 128 threads per SM more warps cost more than they save (300
 // patches of 5^3: 6.4 us at 128 threads, 8.3 at 256).
-inline int untuned_nt(const fv_batch* h, int p, int64_t count, bool known) {
+inline int untuned_nt(const fv_batch* h, int p, int64_t count) {
   int nt = default_nt(h->d, p);
   if (h->d == 1) return nt;
   if (h->prec == FV_FP64) {
     if (h->d == 3 && p == 4) nt = 64;
-    if (h->d == 2 && p >= 9) nt = p <= 12 ? 64 : p < (known ? 20 : 23) ? 128 : 256;
+    if (h->d == 2 && p >= 9) nt = p <= 12 ? 64 : p < 20 ? 128 : 256;
   }
   const int64_t room = (int64_t)h->num_sms * (h->prec == FV_FP64 ? 384 : 128);
   while (nt < 256 && nt < patch_faces(h->d, p) && 2 * nt * count <= room) nt *= 2;

@@ -100,7 +100,7 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
         if (done) continue;
       }
       const int pi = lc.pmax < 64 ? lc.pmax : 63;
-      lc.nt = h->cls_nt[pi] > 0 ? h->cls_nt[pi] : untuned_nt(h, lc.pmax, cnt, true);
+      lc.nt = h->cls_nt[pi] > 0 ? h->cls_nt[pi] : untuned_nt(h, lc.pmax, cnt);
       int& bps = h->occ_cache[f][pi][nt_index(lc.nt)];
       int& ns = h->stage_cache[f][pi][nt_index(lc.nt)];
       if (bps == 0 || pi == 63) {  // slot 63: every size from 63 on
@@ -121,9 +121,7 @@ cudaError_t launch_scheduled(fv_batch* h, UpdateLaunch l) {
     cudaError_t e = launch_one_size(h, lu, l.n, &done);
     if (e != cudaSuccess || done) return e;
   }
-  // whether every patch has the size that the launch is carved for
-  const bool known = plan_ok && h->ncls == 1 && h->cls_real[0] && h->cls_p[0] == h->max_patch_size;
-  l.nt = untuned_nt(h, h->max_patch_size, l.n, known);
+  l.nt = untuned_nt(h, h->max_patch_size, l.n);
   int& bps = h->blocks_per_sm[f][nt_index(l.nt)];
   int& ns = h->nstage[f][nt_index(l.nt)];
   if (bps == 0) {

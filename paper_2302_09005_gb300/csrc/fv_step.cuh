@@ -549,12 +549,13 @@ __host__ __device__ constexpr bool kLoopSums() {
 // threads, sized for a larger patch, a cell's chain of S fixed-point sums leaves
 // most threads idle.  Patches of at most half as many cells as threads; 4 M cells
 // of 2^3 in a handle for 8^3, update 10.0 -> 7.5 ms (for 6^3 4.63 -> 3.60), 4^3
-// 2.40 -> 2.16; mixes of 2^3..8^3 1.54 -> 1.51.  Time steps gain as much there
-// (12.1 -> 10.6 ms) but their code grows by more: 930 patches of 6^3 66 -> 68 us, so
-// they keep the one form.
+// 2.40 -> 2.16; mixes of 2^3..8^3 1.54 -> 1.51; 6 M cells of 5x5 in a handle for 20x20
+// 2.89 -> 2.54, 10x10 1.13 -> 1.05.  Time steps gain as much (2^3 12.1 -> 10.6 ms) but
+// their code grows by more: 930 patches of 6^3 66 -> 68 us, so they keep the one
+// form.
 template <typename T, int D, int P, bool FUSED, int NT>
 __host__ __device__ constexpr bool kItemSums() {
-  return sizeof(T) == 8 && D == 3 && P == 0 && NT == 256 && !FUSED;
+  return sizeof(T) == 8 && D >= 2 && P == 0 && NT == 256 && !FUSED;
 }
 // A patch's state box: read only, but an FP64 time step passes a cell's new state
 // from the loop of its sums to its primitives through it.

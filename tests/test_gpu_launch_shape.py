@@ -1,7 +1,6 @@
-"""CTA sizes that launches really take, read from a captured graph of one call:
-where the sizes of a batch are not known (no plan), a handle for larger 2D
-patches does not take a CTA size that its smaller ones lose by; a class whose
-CTA size was set goes back to the launch's own choice with 0."""
+"""CTA sizes that FP64 launches really take, read from a captured graph of one
+call: a launch per size goes by that size, one launch by the handle's largest;
+a class whose CTA size was set goes back to the launch's own choice with 0."""
 import ctypes
 
 import numpy as np
@@ -69,20 +68,16 @@ def fv():
     return fvmod
 
 
-@pytest.mark.parametrize("pmax,threads", [(12, 64), (19, 128), (20, 128), (22, 128), (23, 256)])
-def test_unknown_sizes(fv, pmax, threads):
-    b, _, stream, call = batch(fv, 2, 5, 3000, pmax)
-    assert kernel_threads(stream, call) == [threads]
-    b.close()
-
-
-@pytest.mark.parametrize("p,threads", [(12, 64), (19, 128), (20, 256), (22, 256)])
-@pytest.mark.parametrize("classes", [True, False])
-def test_known_sizes(fv, p, threads, classes):
-    b, tsz, stream, call = batch(fv, 2, p, 1000, p)
-    fv.fv_batch_plan(b.h, tsz, 1000)
-    if classes:
-        fv.fv_batch_set_schedule(b.h, fv.FV_SCHED_CLASSES)
+@pytest.mark.parametrize("p,pmax,threads", [(5, 12, 64), (5, 19, 128), (5, 20, 256), (12, 12, 64),
+                                            (19, 19, 128), (20, 20, 256)])
+@pytest.mark.parametrize("schedule", [None, 0, 2])  # no plan, one launch, a launch per size
+def test_own_choice(fv, p, pmax, threads, schedule):
+    b, tsz, stream, call = batch(fv, 2, p, 3000, pmax)
+    if schedule is not None:
+        fv.fv_batch_plan(b.h, tsz, 3000)
+        fv.fv_batch_set_schedule(b.h, schedule)
+    if schedule == 2 and p == 5:
+        threads = 32  # the class's own size
     assert kernel_threads(stream, call) == [threads]
     b.close()
 
