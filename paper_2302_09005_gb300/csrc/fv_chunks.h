@@ -9,7 +9,12 @@
 
 namespace fv {
 
-// Bytes of a chunk: on pinned memory an eighth of the batch, 4 to 256 MB.  The
+constexpr int64_t kChunkMin = 4ll << 20, kChunkMax = 256ll << 20;
+
+// Bytes of a chunk: on pinned memory an eighth of the batch, rounded up to whole
+// patches (eight chunks hold it: a ninth of a few patches costs as much as any;
+// no further, since chunks of 1,025 patches of 17x17 copied 5 % slower than the
+// better aligned ones of 1,024), 4 to 256 MB.  The
 // copy in, the update and the copy out overlap only from chunk to chunk, and a
 // chunk costs the host some 20 us.  One chunk / eighths, us per call: 94.6 MB (8,192 2D
 // patches of 17x17, FP64) 1299 / 876, 31.4 MB 660 / 596, 450 MB 4591 / 2847;
@@ -18,9 +23,9 @@ namespace fv {
 // not overlap, so there only the cost of a chunk is left: 256 MB always (256 MB /
 // eighths, us per call in place: 5.9 MB 123 / 164, 56 MB 608 / 1131, 94.6 MB 1237 /
 // 1566, 450 MB 4331 / 4826).
-inline int64_t chunk_bytes(int64_t batch_bytes, bool pinned) {
-  const int64_t lo = 4ll << 20, hi = 256ll << 20, want = pinned ? batch_bytes / 8 : hi;
-  return want < lo ? lo : want > hi ? hi : want;
+inline int64_t chunk_bytes(int64_t batch_bytes, int64_t patch_bytes, bool pinned) {
+  const int64_t want = pinned ? batch_bytes / 8 + patch_bytes - 1 : kChunkMax;
+  return want < kChunkMin ? kChunkMin : want > kChunkMax ? kChunkMax : want;
 }
 
 // The patch after the last one of the chunk that starts at p0: as many as

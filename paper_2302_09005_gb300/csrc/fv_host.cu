@@ -182,9 +182,15 @@ fv_status fv_patch_update_host(fv_batch* h, const void* host_in, void* host_out,
   const bool inplace = host_in == host_out;
   // chunks of chunk_patches patches, or by bytes
   int64_t want = 0;
-  if (chunk_patches <= 0)
-    want = fv::chunk_bytes((off[n - 1] + len(n - 1) - off[0]) * (int64_t)es,
-                           copies_async(host_in) && copies_async(host_out));
+  if (chunk_patches <= 0) {
+    int64_t box = s;  // the largest patch's
+    for (int m = 0; m < d; ++m) box *= h->max_patch_size + 2;
+    const int64_t bytes = (off[n - 1] + len(n - 1) - off[0]) * (int64_t)es;
+    // (a batch of one chunk either way is not looked up)
+    const bool pinned = bytes <= fv::kChunkMin ||
+                        (copies_async(host_in) && (inplace || copies_async(host_out)));
+    want = fv::chunk_bytes(bytes, box * (int64_t)es, pinned);
+  }
   auto end_of = [&](int64_t p0) -> int64_t {
     if (chunk_patches > 0) return n - p0 < chunk_patches ? n : p0 + chunk_patches;
     return fv::chunk_end(p0, n, off, len, (int64_t)es, want);

@@ -12,7 +12,9 @@ from paper_2302_09005_gb300 import _build
 
 SRC = """
 #include "fv_chunks.h"
-extern "C" int64_t bytes_of(int64_t b, int pinned) { return fv::chunk_bytes(b, pinned != 0); }
+extern "C" int64_t bytes_of(int64_t b, int64_t box, int pinned) {
+  return fv::chunk_bytes(b, box, pinned != 0);
+}
 extern "C" int64_t end_of(int64_t p0, int64_t n, const int64_t* off, const int64_t* len, int64_t es,
                           int64_t want) {
   return fv::chunk_end(p0, n, off, [&](int64_t i) { return len[i]; }, es, want);
@@ -29,7 +31,7 @@ def lib(tmp_path_factory):
                     str(d / "t.cpp"), "-o", so], check=True)
     lb = ctypes.CDLL(so)
     lb.bytes_of.restype = lb.end_of.restype = ctypes.c_int64
-    lb.bytes_of.argtypes = [ctypes.c_int64, ctypes.c_int]
+    lb.bytes_of.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int]
     lb.end_of.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p,
                           ctypes.c_int64, ctypes.c_int64]
     return lb
@@ -68,6 +70,24 @@ def test_chunks_by_bytes(lib, kind, gap, want):
 
 def test_chunk_bytes_bounds(lib):
     mb = 1 << 20
-    assert [lib.bytes_of(b, 1) for b in (0, mb, 32 * mb, 80 * mb, 2048 * mb, 1 << 40)] == \
+    sizes = (0, mb, 32 * mb, 80 * mb, 2048 * mb, 1 << 40)
+    assert [lib.bytes_of(b, 1, 1) for b in sizes] == \
         [4 * mb, 4 * mb, 4 * mb, 10 * mb, 256 * mb, 256 * mb]
-    assert [lib.bytes_of(b, 0) for b in (0, 80 * mb, 1 << 40)] == [256 * mb] * 3
+    assert lib.bytes_of(80 * mb, 5, 1) == 10 * mb + 4
+    assert [lib.bytes_of(b, 5, 0) for b in sizes] == [256 * mb] * 6
+
+
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("copies", [3, 7, 8, 9])
+def test_eight_chunks_hold_the_batch(lib, kind, copies):
+    """From 32 MB to 2 GB; patches a little further apart than they are long."""
+    rng = np.random.default_rng(copies)
+    p = np.tile(KINDS[kind](rng), copies * (1000 if kind == "one" else 3)).astype(np.int64)
+    ln = (p + 2) ** 3 * 5
+    off = np.r_[0, np.cumsum(ln + 1)[:-1]].astype(np.int64)
+    total = int(off[-1] + ln[-1]) * 8
+    want = lib.bytes_of(total, 10 ** 3 * 5 * 8, 1)
+    c = cut(lib, off, ln, 8, want)
+    assert total < 2 << 30 and (want == 4 << 20 or len(c) - 1 <= 8)
+    if kind == "uniform":
+        assert c[1] == -(-len(p) // 8)
