@@ -183,8 +183,8 @@ static_assert(kFaceSrcOff + 2 * 6 * (int)sizeof(FaceSrc) <= kHdrBytes, "header t
 // follow the stages.
 // Primitives that are computed, not copied, are the current patch's alone: in
 // FP64 3D CTAs of 256 threads they follow the stages once, and two stages of 8^3
-// fit (4 M cells, step: 8^3 1093 -> 1011 us, 4^3 in a handle for 8^3 2816 -> 2442,
-// update 2179 -> 1914).  Elsewhere two stages fit as it is; smaller CTAs would
+// fit (4 M cells, step: 8^3 1093 -> 997 us, 4^3 in a handle for 8^3 2816 -> 2435,
+// update 2179 -> 1912).  Elsewhere two stages fit as it is; smaller CTAs would
 // only pay for the addresses (2^3, a warp, 1378 -> 1392 us), and in 2D take two
 // stages where one makes as many CTAs resident (2x2 .. 6x6 2.10 -> 2.24 ms).
 template <typename T, int D, int CARRY, int NT>
@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<T, NT>()))
   auto stage_at = [&](int s) -> Stage<T> {
     T* b = sbase + (single ? 0 : s) * cv.stage;
     if constexpr (once) {
-      T* ip = single ? b + cv.box : sbase + 2 * cv.stage;
+      T* ip = sbase + cv.nstage * cv.stage;  // after the stages
       return Stage<T>{b, ip, ip + cv.ip};
     } else {
       return Stage<T>{b, b + cv.box, b + cv.box + cv.ip};
